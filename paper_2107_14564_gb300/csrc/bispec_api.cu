@@ -228,7 +228,7 @@ bsp_status plan_passes(bsp_plan* p, const void* spec, void* fields, cudaStream_t
   if (p->dim == 2) {  // 2D rings: X pass, then the C2R along y on its rows (the Y stage is empty)
     a.st = p->st_full;
     a.items = p->d_xi;
-    if ((st = launch_ring_xpass<T>(a, p->nxi, p->lines_xy, s)) != BSP_OK) return st;
+    if ((st = launch_ring_xpass<T>(a, p->nxi, p->lines.x, s)) != BSP_OK) return st;
     if (ev) {
       BSP_CUDA(cudaEventRecord(ev[0], s));
       BSP_CUDA(cudaEventRecord(ev[1], s));
@@ -238,18 +238,18 @@ bsp_status plan_passes(bsp_plan* p, const void* spec, void* fields, cudaStream_t
     a.g2 = p->g1;
     a.slab_x0 = 0;
     a.slab_nx = 1;
-    if ((st = launch_zpass<T>(a, p->nzi, p->lines_z, s)) != BSP_OK) return st;
+    if ((st = launch_zpass<T>(a, p->nzi, p->lines.z, s)) != BSP_OK) return st;
     if (ev) BSP_CUDA(cudaEventRecord(ev[2], s));
     return BSP_OK;
   }
   if (part < 0) {
     a.st = p->st_full;
     a.items = p->d_xi;
-    st = launch_xpass<T>(a, p->nxi, p->lines_xy, s);
+    st = launch_xpass<T>(a, p->nxi, p->lines.x, s);
     if (st != BSP_OK) return st;
     if (ev) BSP_CUDA(cudaEventRecord(ev[0], s));
     a.items = p->d_yi;
-    st = launch_ypass<T>(a, p->nyi, p->lines_xy, s);
+    st = launch_ypass<T>(a, p->nyi, p->lines.y, s);
     if (st != BSP_OK) return st;
     if (ev) BSP_CUDA(cudaEventRecord(ev[1], s));
     if (part == kPassXY) return BSP_OK;
@@ -264,7 +264,7 @@ bsp_status plan_passes(bsp_plan* p, const void* spec, void* fields, cudaStream_t
   }
   a.st = p->st_half;
   if (split) a.fields = p->fields32;
-  st = launch_zpass<T>(a, nzi, p->lines_z, s);
+  st = launch_zpass<T>(a, nzi, p->lines.z, s);
   if (st != BSP_OK) return st;
   if (split) {
     st = launch_split_fields(static_cast<const float*>(p->fields32), static_cast<uint32_t*>(fields),
@@ -429,7 +429,7 @@ bsp_status ball_setup(bsp_plan* p, cudaStream_t s) {
   ball[0].g1_off = 0;
   ball[0].g2_off = 0;
   std::vector<Item> bx, by, bz;
-  make_items_g(ball, p->ng, warp_fft_lines(), 1, bx, by, bz);
+  make_items_g(ball, p->ng, {warp_fft_lines(), warp_fft_lines(), 1}, bx, by, bz);
   p->nbxi = (int)bx.size();
   p->nbyi = (int)by.size();
   if ((st = dev_upload(p, ball, &p->d_ball, s)) != BSP_OK) return st;

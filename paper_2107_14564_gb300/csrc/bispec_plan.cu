@@ -45,8 +45,29 @@ int fft_lines_for(int len, int prec) {
   return l < 1 ? 1 : l;
 }
 
+// Lines per block of the generic passes: as many as a block holds, fewer where a pass has too few lines
+// to give every SM a block that way, but at least 4 (2 in the Z pass, whose lines are contiguous) so
+// that accesses along k_z keep whole sectors. A 15-ring estimate at Ng = 384 (15 blocks of up to 31 x
+// 96 points a pass before) went from 51.5 to 37.6 us; two, four and eight blocks per SM gave
+// 43.7, 53.2 and 60.2 us, since a block of few lines takes as long as one of some more.
+static int spread(long long lines, int most, int least, int n_sm) {
+  return (int)std::min<long long>(most, std::max<long long>(least, (lines + n_sm - 1) / n_sm));
+}
+
+PassLines pass_lines(const bsp_plan* p, int prec) {
+  const int most = fft_lines_for(p->ngs, prec), most_z = fft_lines_for(p->ngs / 2, prec);
+  long long x = 0, y = 0, z = 0;
+  for (const ShellGeom& g : p->geom) {
+    x += p->dim == 2 ? g.r : (long long)g.r * g.r * 3 / 2;  // lines (k_y, k_z >= 0) that meet the ball
+    y += (long long)p->ngs * g.r;
+    z += p->dim == 2 ? p->ngs : (long long)p->ngs * p->ngs;
+  }
+  const int n_sm = std::max(1, p->n_sm);
+  return {spread(x, most, 4, n_sm), spread(y, most, 4, n_sm), spread(z, most_z, 2, n_sm)};
+}
+
 // Work items of the three passes for shells `geom` on a grid of side `grid`.
-void make_items_g(const std::vector<ShellGeom>& geom, int grid, int lines_xy, int lines_z,
+void make_items_g(const std::vector<ShellGeom>& geom, int grid, const PassLines& lines,
                   std::vector<Item>& xi, std::vector<Item>& yi, std::vector<Item>& zi) {
   const int ng = grid;
   xi.clear(); yi.clear(); zi.clear();
@@ -56,28 +77,28 @@ void make_items_g(const std::vector<ShellGeom>& geom, int grid, int lines_xy, in
     for (int ky = -(r - 1); ky <= r - 1; ++ky) {
       const long long rem = (long long)g.qhi - 1 - (long long)ky * ky;
       const int kzmax = (int)isqrt_ll(rem) + 1;  // kz with ky^2 + kz^2 < qhi
-      for (int kz0 = 0; kz0 < kzmax; kz0 += lines_xy)
-        xi.push_back({n, ky, kz0, std::min(lines_xy, kzmax - kz0)});
+      for (int kz0 = 0; kz0 < kzmax; kz0 += lines.x)
+        xi.push_back({n, ky, kz0, std::min(lines.x, kzmax - kz0)});
     }
     for (int x = 0; x < ng; ++x)
-      for (int kz0 = 0; kz0 < r; kz0 += lines_xy) yi.push_back({n, x, kz0, std::min(lines_xy, r - kz0)});
+      for (int kz0 = 0; kz0 < r; kz0 += lines.y) yi.push_back({n, x, kz0, std::min(lines.y, r - kz0)});
     for (int x = 0; x < ng; ++x)
-      for (int y0 = 0; y0 < ng; y0 += lines_z) zi.push_back({n, x, y0, std::min(lines_z, ng - y0)});
+      for (int y0 = 0; y0 < ng; y0 += lines.z) zi.push_back({n, x, y0, std::min(lines.z, ng - y0)});
   }
 }
 
-void make_items(const bsp_plan* p, int lines_xy, int lines_z, std::vector<Item>& xi,
+void make_items(const bsp_plan* p, const PassLines& lines, std::vector<Item>& xi,
                 std::vector<Item>& yi, std::vector<Item>& zi) {
   if (p->dim == 2) {  // 2D rings: k_y lines for the X pass (xi), x rows for the C2R along y (zi)
     xi.clear(); yi.clear(); zi.clear();
     for (int n = 0; n < p->ns; ++n) {
       const int r = p->geom[n].r;
-      for (int ky0 = 0; ky0 < r; ky0 += lines_xy) xi.push_back({n, 0, ky0, std::min(lines_xy, r - ky0)});
-      for (int x0 = 0; x0 < p->ngs; x0 += lines_z) zi.push_back({n, 0, x0, std::min(lines_z, p->ngs - x0)});
+      for (int ky0 = 0; ky0 < r; ky0 += lines.x) xi.push_back({n, 0, ky0, std::min(lines.x, r - ky0)});
+      for (int x0 = 0; x0 < p->ngs; x0 += lines.z) zi.push_back({n, 0, x0, std::min(lines.z, p->ngs - x0)});
     }
     return;
   }
-  make_items_g(p->geom, p->ngs, lines_xy, lines_z, xi, yi, zi);
+  make_items_g(p->geom, p->ngs, lines, xi, yi, zi);
 }
 
 // Tiles of up to 4 consecutive pairs x 4 consecutive c over a list of bins sorted by (a, b, c).
@@ -317,7 +338,7 @@ TcGrouping group_pairs(const std::vector<int2>& pairs, int nf, int kt_max) {
 template <typename T>
 bsp_status run_passes(const bsp_plan* p, const void* spec, int rsd, void* tw, void* g1, void* g2,
                       void* fields, const Item* xi, int nxi, const Item* yi, int nyi, const Item* zi,
-                      int nzi, int lines_xy, int lines_z, cudaStream_t s, int kweight = 0, bool do_xy = true,
+                      int nzi, const PassLines& lines, cudaStream_t s, int kweight = 0, bool do_xy = true,
                       bool do_z = true, int slab_x0 = 0, int slab_nx = 0) {
   PassArgs a{};
   a.n_sm = p->n_sm;
@@ -336,21 +357,21 @@ bsp_status run_passes(const bsp_plan* p, const void* spec, int rsd, void* tw, vo
   if (p->dim == 2) {  // 2D rings: X pass, then the C2R along y (the Z-pass kernel on its rows)
     a.st = p->st_full;
     a.items = xi;
-    if ((st = launch_ring_xpass<T>(a, nxi, lines_xy, s)) != BSP_OK) return st;
+    if ((st = launch_ring_xpass<T>(a, nxi, lines.x, s)) != BSP_OK) return st;
     a.items = zi;
     a.st = p->st_half;
     a.g2 = g1;
     a.slab_x0 = 0;
     a.slab_nx = 1;
-    return launch_zpass<T>(a, nzi, lines_z, s);
+    return launch_zpass<T>(a, nzi, lines.z, s);
   }
   if (do_xy) {
     a.st = p->st_full;
     a.items = xi;
-    st = launch_xpass<T>(a, nxi, lines_xy, s);
+    st = launch_xpass<T>(a, nxi, lines.x, s);
     if (st != BSP_OK) return st;
     a.items = yi;
-    st = launch_ypass<T>(a, nyi, lines_xy, s);
+    st = launch_ypass<T>(a, nyi, lines.y, s);
     if (st != BSP_OK) return st;
   }
   if (!do_z) return BSP_OK;
@@ -358,7 +379,7 @@ bsp_status run_passes(const bsp_plan* p, const void* spec, int rsd, void* tw, vo
   a.st = p->st_half;
   a.slab_x0 = slab_x0;
   a.slab_nx = slab_nx;
-  return launch_zpass<T>(a, nzi, lines_z, s);
+  return launch_zpass<T>(a, nzi, lines.z, s);
 }
 
 int pick_gridx_n(int n_sm, int ntiles, long long nvox) {
@@ -913,10 +934,9 @@ bsp_status plan_sums(bsp_plan* p, bool lengths, const std::vector<int>& ca, cons
                      cudaStream_t s) {
   const int nf = lengths ? 2 * p->ns : p->ns + p->n_extra();  // order 4: shell fields, then pair products
   const int S = p->ngs;
-  const int lxy = fft_lines_for(S, BSP_FP64);
-  const int lz = fft_lines_for(S / 2, BSP_FP64);
+  const PassLines lines = pass_lines(p, BSP_FP64);
   std::vector<Item> xi, yi, zi;
-  make_items(p, lxy, lz, xi, yi, zi);
+  make_items(p, lines, xi, yi, zi);
   // under a memory budget the FP64 fields are produced and contracted one x-slab at a time
   int nx = S;
   if (p->mem_budget > 0) {
@@ -948,19 +968,17 @@ bsp_status plan_sums(bsp_plan* p, bool lengths, const std::vector<int>& ca, cons
   TRY(launch_twiddles<double>(tw, S, s));
   if (!slab) {
     TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi,
-                           (int)zi.size(), lxy, lz, s));
+                           (int)zi.size(), lines, s));
     if (p->order == 4)
       TRY(launch_pair_fields<double>(f, slab_vox, p->d_pairs4, p->n_extra(),
                                      static_cast<double*>(f) + (size_t)p->ns * slab_vox, p->n_sm, s));
     if (lengths)
       TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, static_cast<double*>(f) + (size_t)p->ns * slab_vox,
-                             dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, (int)zi.size(), lxy, lz, s, 1));
+                             dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, (int)zi.size(), lines, s, 1));
   } else {
-    TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, 0, lxy,
-                           lz, s, 0, true, false));
+    TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, 0, lines, s, 0, true, false));
     if (lengths)
-      TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, 0, lxy,
-                             lz, s, 1, true, false));
+      TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, 0, lines, s, 1, true, false));
   }
   std::vector<int2> pairs;
   std::vector<Tile> tiles;
@@ -991,11 +1009,11 @@ bsp_status plan_sums(bsp_plan* p, bool lengths, const std::vector<int>& ca, cons
       const int x0 = k * nx, len = std::min(nx, S - x0);
       const int nzk = zoff[k + 1] - zoff[k];
       c.nvox = (long long)len * S * S;
-      TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, 0, dyi, 0, dzi + zoff[k], nzk, lxy, lz, s, 0, false,
+      TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, 0, dyi, 0, dzi + zoff[k], nzk, lines, s, 0, false,
                              true, x0, len));
       if (lengths)
         TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, static_cast<double*>(f) + (size_t)p->ns * c.nvox, dxi, 0,
-                               dyi, 0, dzi + zoff[k], nzk, lxy, lz, s, 1, false, true, x0, len));
+                               dyi, 0, dzi + zoff[k], nzk, lines, s, 1, false, true, x0, len));
     }
     c.accumulate = k > 0;
     TRY(launch_contract_simt<double>(c, s));
@@ -1126,10 +1144,9 @@ bsp_status bsp_plan_create(const bsp_plan_desc* desc, void* stream, bsp_plan** o
     t.inside = (t.t >= 0.5 && t.t <= 1.0 && t.mu >= 0.5 && t.mu <= 1.0 && 2.0 * t.mu * t.t >= 1.0) ? 1 : 0;
   }
   // estimator buffers in the plan's precision
-  p->lines_xy = fft_lines_for(p->ngs, p->prec);
-  p->lines_z = fft_lines_for(p->ngs / 2, p->prec);
+  p->lines = pass_lines(p, p->prec);
   std::vector<Item> xi, yi, zi;
-  make_items(p, p->lines_xy, p->lines_z, xi, yi, zi);
+  make_items(p, p->lines, xi, yi, zi);
   p->nxi = (int)xi.size(); p->nyi = (int)yi.size(); p->nzi = (int)zi.size();
   const size_t ce = p->prec == BSP_FP64 ? sizeof(double2) : sizeof(float2);
   std::vector<int> cptr(p->n_cells() + 1, 0), cidx;
@@ -1161,7 +1178,7 @@ bsp_status bsp_plan_create(const bsp_plan_desc* desc, void* stream, bsp_plan** o
     TRY(dev_upload(p, t1, &p->d_stw, s));
     TRY(dev_upload(p, t2, &p->d_stw_half, s));
     std::vector<Item> wx, wy, wz;
-    make_items(p, warp_fft_lines(), 1, wx, wy, wz);
+    make_items(p, {warp_fft_lines(), warp_fft_lines(), 1}, wx, wy, wz);
     p->nwxi = (int)wx.size();
     p->nwyi = (int)wy.size();
     TRY(dev_upload(p, wx, &p->d_wxi, s));

@@ -30,6 +30,9 @@ inline bool make_stages(int n, FftStages* st) {
   return m == 1;
 }
 
+// Lines per block of the generic X, Y and Z passes.
+struct PassLines { int x, y, z; };
+
 // Device allocation owned by a plan.
 struct DevBuf {
   void* p = nullptr;
@@ -101,7 +104,7 @@ struct bsp_plan {
   std::vector<ShellGeom> geom;
   std::vector<bsp_triplet> trips;  // kept bins
   FftStages st_full{}, st_half{};
-  int lines_xy = 0, lines_z = 0;
+  PassLines lines{};
   int n_sm = 0;
   // device buffers
   std::vector<DevBuf> bufs;
@@ -199,9 +202,10 @@ bsp_status dev_upload(bsp_plan* p, const std::vector<V>& h, V** out, cudaStream_
 }
 
 int fft_lines_for(int len, int prec);
-void make_items_g(const std::vector<ShellGeom>& geom, int grid, int lines_xy, int lines_z,
+PassLines pass_lines(const bsp_plan* p, int prec);
+void make_items_g(const std::vector<ShellGeom>& geom, int grid, const PassLines& lines,
                   std::vector<Item>& xi, std::vector<Item>& yi, std::vector<Item>& zi);
-void make_items(const bsp_plan* p, int lines_xy, int lines_z, std::vector<Item>& xi,
+void make_items(const bsp_plan* p, const PassLines& lines, std::vector<Item>& xi,
                 std::vector<Item>& yi, std::vector<Item>& zi);
 void make_tiles(const std::vector<int>& ta, const std::vector<int>& tb, const std::vector<int>& tc,
                 std::vector<int2>& pairs, std::vector<Tile>& tiles, std::vector<int>& map,
