@@ -49,78 +49,45 @@ template <typename T>
 bsp_status run_contract(bsp_plan* p, const void* fields, double* msum, cudaStream_t s, cudaEvent_t mid,
                         bool levels_ready = false) {
   bsp_status st;
-  // contraction kernels of every level (lower levels first sample their fields)
+  if (p->prec != BSP_MIXED_BF16X3) {
+    SumArgs a = p->sums;
+    a.fields = fields;
+    a.msum = msum;
+    if ((st = launch_contract_simt<T>(a, s)) != BSP_OK) return st;
+    if (mid) BSP_CUDA(cudaEventRecord(mid, s));
+    return launch_reduce_sums(a, s);
+  }
+  // tensor-core kernels of every level (lower levels first sample their fields, unless the split
+  // Z pass wrote them)
   for (ContractLevel& L : p->levels) {
-    const void* f = fields;
-    if (!L.top && levels_ready) {
-      f = L.fields;  // written by the split Z pass
-    } else if (!L.top) {
-      if (p->prec == BSP_MIXED_BF16X3)  // split planes sampled as 2 x shells bf16 fields
-        st = launch_decimate<uint16_t>(fields, p->ngs, L.d_shells, 2 * (int)L.shells.size(), L.fields, L.g, L.stride,
-                                       p->n_sm, s);
-      else
-        st = launch_decimate<T>(fields, p->ngs, L.d_shells, (int)L.shells.size(), L.fields, L.g, L.stride, p->n_sm, s);
+    if (!L.top && !levels_ready) {  // split planes sampled as 2 x shells bf16 fields
+      st = launch_decimate(static_cast<const uint16_t*>(fields), p->ngs, L.d_shells, 2 * (int)L.shells.size(),
+                           static_cast<uint16_t*>(L.fields), L.g, L.stride, p->n_sm, s);
       if (st != BSP_OK) return st;
-      f = L.fields;
     }
-    if (p->prec == BSP_MIXED_BF16X3) {
-      TcArgs a{};
-      a.nvox = L.nvox();
-      a.np = L.np;
-      a.kt = L.kt;
-      a.groups = L.d_tc_groups;
-      a.n_tg = L.n_tg;
-      a.gridy = L.gridy;
-      a.vox_per_block = L.vpb;
-      a.partial = L.tc_partial;
-      a.error = p->d_error;
-      st = launch_contract_tc(a, &L.tmap, s);
-    } else {
-      ContractArgs c{};
-      c.fields = f;
-      c.nvox = L.nvox();
-      c.ns = (int)L.shells.size();
-      c.tiles = L.d_tiles;
-      c.pairs = L.d_pairs;
-      c.tile_map = L.d_map;
-      c.ntiles = L.ntiles;
-      c.gridx = L.gridx;
-      c.partial = L.partial;
-      c.msum = msum;
-      c.n_out = (int)L.bins.size();
-      c.scale = L.scale;
-      st = launch_contract_simt<T>(c, s);
-    }
-    if (st != BSP_OK) return st;
+    TcArgs a{};
+    a.nvox = L.nvox();
+    a.np = L.np;
+    a.kt = L.kt;
+    a.groups = L.d_tc_groups;
+    a.n_tg = L.n_tg;
+    a.gridy = L.gridy;
+    a.vox_per_block = L.vpb;
+    a.partial = L.tc_partial;
+    a.error = p->d_error;
+    if ((st = launch_contract_tc(a, &L.tmap, s)) != BSP_OK) return st;
   }
   if (mid) BSP_CUDA(cudaEventRecord(mid, s));
   // cross-block sums of every level, scaled to the ng^3 grid
-  if (p->prec == BSP_MIXED_BF16X3) return launch_reduce_tc_all(p->d_tc_bins, (int)p->trips.size(), msum, s);
-  for (ContractLevel& L : p->levels) {
-    {
-      ContractArgs c{};
-      c.tile_map = L.d_map;
-      c.ntiles = L.ntiles;
-      c.gridx = L.gridx;
-      c.partial = L.partial;
-      c.msum = msum;
-      c.scale = L.scale;
-      st = launch_reduce_partials(c, s);
-    }
-    if (st != BSP_OK) return st;
-  }
-  return BSP_OK;
+  return launch_reduce_tc_all(p->d_tc_bins, (int)p->trips.size(), msum, s);
 }
 
 // Kernels launched by run_contract.
 int contract_launches(const bsp_plan* p) {
-  int n = 0;
-  for (const ContractLevel& L : p->levels) {
-    const bool work = p->prec == BSP_MIXED_BF16X3 ? L.n_tg > 0 : L.ntiles > 0;
-    const bool sampled = !L.top && !(p->prec == BSP_MIXED_BF16X3 && p->n_zlev > 0);  // else the Z pass did it
-    n += sampled + (p->prec == BSP_MIXED_BF16X3 ? 1 : 2) * work;
-  }
-  return n + (p->prec == BSP_MIXED_BF16X3 ? 1 : 0);  // one cross-block sum for all tensor-core levels
+  if (p->prec != BSP_MIXED_BF16X3) return 2 * (p->sums.items > 0);
+  int n = 1;  // one cross-block sum for all tensor-core levels
+  for (const ContractLevel& L : p->levels) n += (!L.top && p->n_zlev == 0) + (L.n_tg > 0);
+  return n;
 }
 
 // The contraction of x-slab k of an x-slab plan (one level, the evaluation grid) on the slab's
@@ -128,10 +95,12 @@ int contract_launches(const bsp_plan* p) {
 template <typename T>
 bsp_status contract_slab(bsp_plan* p, int k, cudaStream_t s) {
   if (p->levels.empty()) return BSP_OK;
-  const ContractLevel& L = p->levels[0];
+  const bool last = k == p->n_slabs() - 1 && p->slab_len(k) != p->slab_len(0);
+  bsp_status st;
   if (p->prec == BSP_MIXED_BF16X3) {
     // the slab's split fields through the full-slab or last-slab tensor map, a fixed number of
     // voxel blocks (blocks past the slab's voxels write zero sums), sums added over the slabs
+    const ContractLevel& L = p->levels[0];
     if (L.n_tg == 0) return BSP_OK;
     const long long nvox = (long long)p->slab_len(k) * p->ngs * p->ngs;
     const long long chunks = nvox / kTcVoxelChunk;
@@ -145,29 +114,16 @@ bsp_status contract_slab(bsp_plan* p, int k, cudaStream_t s) {
     a.vox_per_block = ((chunks + L.gridy - 1) / L.gridy) * kTcVoxelChunk;
     a.partial = L.tc_partial;
     a.error = p->d_error;
-    const bool last = k == p->n_slabs() - 1 && p->slab_len(k) != p->slab_len(0);
-    bsp_status st = launch_contract_tc(a, last ? &L.tmap_last : &L.tmap, s);
+    st = launch_contract_tc(a, last ? &L.tmap_last : &L.tmap, s);
     if (st != BSP_OK) return st;
     return launch_reduce_tc_all(p->d_tc_bins, (int)p->trips.size(), p->msum, s, k > 0);
   }
-  if (L.ntiles == 0) return BSP_OK;
-  ContractArgs c{};
-  c.fields = p->fields;
-  c.nvox = (long long)p->slab_len(k) * p->ngs * p->ngs;
-  c.ns = p->ns;
-  c.tiles = L.d_tiles;
-  c.pairs = L.d_pairs;
-  c.tile_map = L.d_map;
-  c.ntiles = L.ntiles;
-  c.gridx = L.gridx;
-  c.partial = L.partial;
-  c.msum = p->msum;
-  c.n_out = (int)L.bins.size();
-  c.scale = L.scale;
-  c.accumulate = k > 0;
-  bsp_status st = launch_contract_simt<T>(c, s);
-  if (st != BSP_OK) return st;
-  return launch_reduce_partials(c, s);
+  SumArgs a = last ? p->sums_last : p->sums;
+  a.fields = p->fields;
+  a.msum = p->msum;
+  a.accumulate = k > 0;
+  if ((st = launch_contract_simt<T>(a, s)) != BSP_OK) return st;
+  return launch_reduce_sums(a, s);
 }
 
 // The pass launches of an estimate on the plan's buffers; ev (optional) receives an event after
@@ -326,7 +282,7 @@ bsp_status estimate_impl(bsp_plan* p, const void* spec, double* b_trip, double* 
       int passes = p->warp_fft ? 2 + p->n_slabs() : (p->nxi > 0) + (p->nyi > 0);
       if (!p->warp_fft)
         for (int k = 0; k < p->n_slabs(); ++k) passes += p->zi_off[k + 1] > p->zi_off[k];
-      const bool work = !p->levels.empty() && (split ? p->levels[0].n_tg > 0 : p->levels[0].ntiles > 0);
+      const bool work = !p->levels.empty() && (split ? p->levels[0].n_tg > 0 : p->sums.items > 0);
       p->launches += passes + 2LL * work * p->n_slabs() + 1;
     } else {
       const int passes = (p->warp_fft ? 3 : (p->nxi > 0) + (p->nyi > 0) + (p->nzi > 0) + (split ? 1 : 0)) +

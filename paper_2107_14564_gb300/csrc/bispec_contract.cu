@@ -1,14 +1,26 @@
 // Triple-product reduction on CUDA cores and the final normalisation.
 //
 // msum[t] = sum_x d_a(x) d_b(x) d_c(x) for every kept bin t = (a, b, c) (numerator of Eq. (2.7);
-// with counting fields, the T_abc of Eq. (2.10)). The bins are grouped as
-// M[(a,b), c] = sum_x (d_a d_b)(x) d_c(x): a tile owns up to 4 pairs (a, b) and 4 consecutive
-// c, i.e. 16 outputs held in registers by one thread. A block walks a contiguous voxel range in
-// chunks staged in shared memory (all shells of the chunk), so every field value read from
-// HBM serves every tile of the block; the next chunk is copied in with cp.async into a second
-// buffer while the current one is used. FP32 plans accumulate in FP32 over kFlushChunks chunks
-// and then add into FP64; FP64 plans accumulate in FP64. Blocks write FP64 partial sums,
-// which a second kernel adds in a fixed order (deterministic results).
+// with counting fields, the T_abc of Eq. (2.10)). One launch sums the bins of every contraction
+// level, sampling the coarser levels' voxels from the evaluation grid's fields with their stride;
+// a second adds the partial sums in FP64 in a fixed order (deterministic results).
+//
+// FP32: an output's products are added in voxel order over runs of kSumRun voxels, the runs in
+// FP64. A lane owns one run and a warp one tile of 2 x 4 x 8 outputs (a, b, c), so 32 runs go
+// through the same 8 pair products and 64 multiply-adds per voxel and no lane idles for want of bins;
+// tiles at the edge of the triangle region take 2 b or 4 c.
+//   * What bounds it: the FMA units (at most 67% of their rate with three register reads each,
+//     measured on an outer product), then the warps' waits at the stages' barriers. Shared memory
+//     delivers 32 words per cycle whatever lanes share (measured: LDS.128 takes 4 cycles a warp even
+//     when its lanes read 8 distinct quads), so a tile has to use a word often: 2 x 4 x 8 reads 14
+//     words a voxel for 72 operations, 2 x 4 x 4 reads 10 for 40, 1 x 4 x 4 reads 9 for 20.
+//   * Also measured at Ng = 256 and 24 shells: two runs packed in a lane's registers (1.38 ms), tiles
+//     in threads with lanes on different tiles of one voxel (1.36); the earlier layout was of that
+//     kind with 1 x 4 x 4 tiles, 118 of 256 threads in use.
+// FP64 (1/64 of the FP32 rate: 2 multiply-adds per SM and cycle): any order of additions will do,
+// so lanes own voxels and a warp exactly the pair products and multiply-adds its bins need, none
+// for tile padding; loads go straight to L1. Ng = 128 and 16 shells 2.43 -> 1.04 ms, Ng = 32 and 8
+// shells 46.6 -> 13.1 us (there the earlier blocks summed 64 voxels in 11 threads).
 #include <algorithm>
 
 #include "common.cuh"
@@ -16,154 +28,358 @@
 
 namespace bsp {
 
-constexpr int kChunk = 64;         // voxels per shared-memory chunk
-constexpr int kContractThreads = 256;
-constexpr int kFlushChunks = 16;   // FP32 run length: 1024 voxels
+namespace {
 
-// Two neighbouring voxels of one field, read from shared memory in one 8-byte (FP32) or
-// 16-byte (FP64) load.
-template <typename T> struct Pair2;
-template <> struct Pair2<float> { using type = float2; };
-template <> struct Pair2<double> { using type = double2; };
-// Row stride of a staged chunk: even, so voxel pairs are aligned; 66 words puts field n's pair
-// (v, v + 1) on the bank pair (n + v / 2) mod 16.
-constexpr int kChunkLd = kChunk + 2;
+constexpr int kSumThreads = 32 * kSumWarps;
+constexpr int kSumVox = 32;     // voxels of a run per stage: whole cache lines
+constexpr int kSumQuads = kSumVox / 4;
+constexpr int kSumRow = 4 * kSumVox;          // bytes of a run in a staged field
+constexpr int kSumFieldBytes = 32 * kSumRow;  // one field of a stage: 32 runs
+// Run r's quad q lies in place q ^ sum_swz(r): eight lanes' 16-byte reads of one field meet all banks.
+__host__ __device__ constexpr int sum_swz(int r) {
+  return (r >> (kSumVox == 8 ? 2 : kSumVox == 16 ? 1 : 0)) & (kSumQuads - 1);
+}
+constexpr int kF64Warps = 4;
+constexpr int kF64Run = 64;  // 32-voxel steps summed lane by lane
 
-template <typename T>
-__global__ void __launch_bounds__(kContractThreads)
-contract_simt_kernel(ContractArgs a, long long vox_per_block) {
-  using T2 = typename Pair2<T>::type;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* dsm0 = reinterpret_cast<T*>(smem_raw);  // two chunks [ns][kChunkLd]
-  constexpr int LD = kChunkLd;
-  const int chunk_elems = a.ns * LD;
-  const T* fields = static_cast<const T*>(a.fields);
-  const int tile = blockIdx.y * kContractThreads + threadIdx.x;
-  const bool active = tile < a.ntiles;
-  int ia[4], ib[4], c0 = 0;
+// The level of work item w.
+__device__ __forceinline__ const SumLevel& level_of(const SumArgs& a, int w) {
+  int l = 0;
+  while (l + 1 < a.n_lv && w >= a.lv[l + 1].w0) ++l;
+  return a.lv[l];
+}
+
+// Lane l ends with the sum over the warp of its v[l]: halves are exchanged, so 31 additions in
+// all instead of 5 per output.
+__device__ __forceinline__ double warp_transpose_sum(const float* v, int lane) {
+  double d[16];
+  {
+    const bool up = (lane & 16) != 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { ia[i] = 0; ib[i] = 0; }
-  if (active) {
-    const Tile t = a.tiles[tile];
-    c0 = t.c0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int p = t.p0 + (i < t.np ? i : 0);
-      const int2 ab = a.pairs[p];
-      ia[i] = ab.x;
-      ib[i] = ab.y;
+    for (int i = 0; i < 16; ++i) {
+      const float send = up ? v[i] : v[i + 16];
+      const float keep = up ? v[i + 16] : v[i];
+      d[i] = (double)keep + (double)__shfl_xor_sync(0xffffffffu, send, 16);
     }
   }
-  int ic[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) ic[j] = min(c0 + j, a.ns - 1);
-
-  double acc64[16];
-  T acc[16];
+  for (int o = 8; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) { acc64[k] = 0.0; acc[k] = T(0); }
+    for (int i = 0; i < o; ++i) {
+      const double send = up ? d[i] : d[i + o];
+      const double keep = up ? d[i + o] : d[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return d[0];
+}
+__device__ __forceinline__ double warp_transpose_sum(const double* v, int lane) {
+  double d[16];
+  {
+    const bool up = (lane & 16) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const double send = up ? v[i] : v[i + 16];
+      const double keep = up ? v[i + 16] : v[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double send = up ? d[i] : d[i + o];
+      const double keep = up ? d[i + o] : d[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return d[0];
+}
 
-  const long long v_begin = (long long)blockIdx.x * vox_per_block;
-  const long long v_end = min(v_begin + vox_per_block, a.nvox);
-  // copy the chunk at vb into dst (zeros past v_end), one commit group
-  auto stage = [&](long long vb, T* dst) {
-    for (int i = threadIdx.x; i < a.ns * kChunk; i += kContractThreads) {
-      const int n = i / kChunk;
-      const int v = i - n * kChunk;
-      const long long gv = vb + v;
-      const bool in = gv < v_end;
-      ptx::cp_async_zfill<(int)sizeof(T)>(dst + n * LD + v, in ? fields + (long long)n * a.nvox + gv : fields,
-                                          in ? (uint32_t)sizeof(T) : 0u);
+// ---------------------------------------------------------------- FP32
+// Four voxels of this lane's row of a staged field: one 16-byte load.
+__device__ __forceinline__ void lds_quad(uint32_t addr, float (&v)[4]) {
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(addr));
+}
+
+// One quad of a tile whose fields are in registers: two neighbouring voxels' pair products are one
+// packed multiplication; their triple products are added in voxel order.
+template <int NB, int NC>
+__device__ __forceinline__ void sum_quad(const float (&a)[2][4], const float (&b)[NB][4], const float (&c)[NC][4],
+                                         float (&acc)[64]) {
+#pragma unroll
+  for (int h = 0; h < 4; h += 2) {
+    uint64_t p[2][NB];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < NB; ++j)
+        p[i][j] = ptx::f2_mul(ptx::f2_pack(a[i][h], a[i][h + 1]), ptx::f2_pack(b[j][h], b[j][h + 1]));
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+          const float x = __uint_as_float((uint32_t)(e ? p[i][j] >> 32 : p[i][j]));
+#pragma unroll
+          for (int k = 0; k < NC; ++k) acc[32 * i + 8 * j + k] = fmaf(x, c[k][h + e], acc[32 * i + 8 * j + k]);
+        }
+  }
+}
+
+// A stage, two quads at a time: the second's loads are under way while the first is summed. A, B, C
+// are the shared-memory addresses of this lane's row of the tile's fields, swz the exchange of its
+// quads (see contract_f32_kernel).
+template <int NB, int NC>
+__device__ __forceinline__ void sum_stage(const uint32_t (&A)[2], const uint32_t (&B)[4], const uint32_t (&C)[8],
+                                          uint32_t off, uint32_t swz, float (&acc)[64]) {
+#pragma unroll 1
+  for (uint32_t q = 0; q < kSumVox * 4; q += 32) {
+    float a[2][2][4], b[2][NB][4], c[2][NC][4];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const uint32_t o = off + ((q + 16 * t) ^ swz);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) lds_quad(A[i] + o, a[t][i]);
+#pragma unroll
+      for (int i = 0; i < NB; ++i) lds_quad(B[i] + o, b[t][i]);
+#pragma unroll
+      for (int i = 0; i < NC; ++i) lds_quad(C[i] + o, c[t][i]);
+    }
+    sum_quad<NB, NC>(a[0], b[0], c[0], acc);
+    sum_quad<NB, NC>(a[1], b[1], c[1], acc);
+  }
+}
+
+// Block = (level, sub, group of 32 runs). A stage holds kSumVox voxels of every run of the group
+// for the sub's fields, [field][run][voxel], the quads of a run exchanged so that eight lanes' 16-byte
+// reads of one field meet all banks. 128 bytes a run and stage: a copy that brings less than a
+// cache line still occupies shared memory for a cycle (8 voxels a stage: 1.45 ms, 16: 1.25, 32:
+// 1.13, at Ng = 256 and 24 shells). One block of 8 warps an SM, two stages of up to 27 fields.
+__global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ long long foff[kSumMaxFields];
+  const int tid = threadIdx.x;
+  const int lane = tid & 31;
+  const SumLevel L = level_of(a, blockIdx.x);
+  const int unit = (int)(blockIdx.x - L.w0);
+  const int grp = unit / L.units;  // the subs of a group run side by side: its fields stay in L2
+  const SumSub sub = L.subs[unit - grp * L.units];
+  const float* fields = static_cast<const float*>(a.fields);
+  if (tid < sub.nf) foff[tid] = (long long)L.sub_fields[sub.field0 + tid] * L.fstride;
+  // the runs of the group: whole runs first, then the summation blocks' remainders; lane r sums run r
+  const bool whole = grp < L.ngf;
+  const int len = whole ? kSumRun : L.vpb - L.nfull * kSumRun;
+  __shared__ int2 runs[32];
+  if (tid < 32) {
+    const int i = (whole ? grp : grp - L.ngf) * 32 + tid;
+    const int b = whole ? i / L.nfull : i;
+    int2 v = make_int2(0, 0);
+    if (b < L.nblk) {
+      const long long first = (long long)b * L.vpb;
+      const long long start = first + (long long)(whole ? i - b * L.nfull : L.nfull) * kSumRun;
+      const long long end = min(min(first + (long long)L.vpb, L.nvox), start + (long long)len);
+      if (end > start) v = make_int2((int)start, (int)end);
+    }
+    runs[tid] = v;
+  }
+  __syncthreads();
+  // copies: this thread takes quad cq of run cr of every (kSumThreads / 32 kSumQuads)-th field
+  const int stage_bytes = sub.nf * kSumFieldBytes;
+  const int cq = tid % kSumQuads, cr = (tid / kSumQuads) & 31;
+  constexpr int kStep = kSumThreads / (32 * kSumQuads);
+  static_assert(kStep >= 1 && kStep * 32 * kSumQuads == kSumThreads, "a thread copies one quad of one run");
+  const int f0 = tid / (32 * kSumQuads);
+  const int2 run = runs[cr];
+
+  unsigned char* const cdst = smem + cr * kSumRow + ((cq ^ sum_swz(cr)) << 4);
+  auto issue = [&](int k, int buf) {
+    unsigned char* dst = cdst + buf * stage_bytes;
+    const int v = run.x + k * kSumVox + 4 * cq;
+    const bool in = v < run.y;
+    if (L.t == 1) {
+      const float* src = fields + (in ? v : 0);
+      const uint32_t n = in ? 16u : 0u;
+#pragma unroll 4
+      for (int f = f0; f < sub.nf; f += kStep) ptx::cp_async16_zfill(dst + f * kSumFieldBytes, src + foff[f], n);
+    } else {
+      long long o = 0;
+      if (in) {  // g is a multiple of 8: the quad lies in one row of the level's grid
+        const unsigned g = (unsigned)L.g, u = (unsigned)v;
+        const unsigned xy = u / g, z = u - xy * g, x = xy / g, y = xy - x * g;
+        o = ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
+      }
+      const float* src = fields + o;
+      for (int f = f0; f < sub.nf; f += kStep)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 4 * e, in ? src + foff[f] + e * L.t : fields, in ? 4u : 0u);
     }
     ptx::cp_async_commit();
   };
-  if (v_begin < v_end) stage(v_begin, dsm0);
-  int run = 0, k = 0;
-  for (long long vb = v_begin; vb < v_end; vb += kChunk, ++k) {
-    const T* dsm = dsm0 + (size_t)(k & 1) * chunk_elems;
-    if (vb + kChunk < v_end) {
-      stage(vb + kChunk, dsm0 + (size_t)((k + 1) & 1) * chunk_elems);
-      ptx::cp_async_wait<1>();  // this chunk's copies (issued one iteration earlier) have landed
-    } else {
-      ptx::cp_async_wait<0>();
-    }
-    __syncthreads();
+  const int warp = tid >> 5;
+  uint32_t A[2], B[4], C[8];
+  const bool active = warp < sub.ntiles;
+  const uint32_t swz = (uint32_t)sum_swz(lane) << 4;
+  {
+    const SumTile t = L.tiles[sub.tile0 + (active ? warp : 0)];
+    const uint32_t row = ptx::smem_u32(smem) + lane * kSumRow;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) A[i] = row + t.a[i] * kSumFieldBytes;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) B[i] = row + t.b[i] * kSumFieldBytes;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) C[i] = row + t.c[i] * kSumFieldBytes;
+  }
+  float acc[64];
+#pragma unroll
+  for (int i = 0; i < 64; ++i) acc[i] = 0.f;
+  const int nst = len / kSumVox;
+  issue(0, 0);
+  for (int k = 0; k < nst; ++k) {
+    ptx::cp_async_wait<0>();  // stage k has landed
+    __syncthreads();          // for every thread, and stage k - 1 has been read
+    if (k + 1 < nst) issue(k + 1, (k + 1) & 1);
     if (active) {
-#pragma unroll 2
-      for (int v = 0; v < kChunk; v += 2) {  // voxels v and v + 1, added in that order
-        T2 p[4], d[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const T2 x = *reinterpret_cast<const T2*>(dsm + ia[i] * LD + v);
-          const T2 y = *reinterpret_cast<const T2*>(dsm + ib[i] * LD + v);
-          p[i].x = x.x * y.x;
-          p[i].y = x.y * y.y;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) d[j] = *reinterpret_cast<const T2*>(dsm + ic[j] * LD + v);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i * 4 + j] = fma(p[i].x, d[j].x, acc[i * 4 + j]);
-            acc[i * 4 + j] = fma(p[i].y, d[j].y, acc[i * 4 + j]);
-          }
-      }
-      if (++run == kFlushChunks) {
-        run = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) { acc64[q] += (double)acc[q]; acc[q] = T(0); }
+      const uint32_t off = (uint32_t)((k & 1) * stage_bytes);
+      switch (sub.kind) {  // the same for the block's tiles
+        case 3: sum_stage<4, 8>(A, B, C, off, swz, acc); break;
+        case 2: sum_stage<4, 4>(A, B, C, off, swz, acc); break;
+        case 1: sum_stage<2, 8>(A, B, C, off, swz, acc); break;
+        default: sum_stage<2, 4>(A, B, C, off, swz, acc);
       }
     }
-    __syncthreads();  // every thread is done with this buffer before the next copy into it
   }
-  if (active) {  // partial[(tile * 16 + k) * gridx + block]: an output's block sums are contiguous
-    double* out = a.partial + (long long)tile * 16 * a.gridx + blockIdx.x;
+  if (active) {
+    float half[32];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) out[(long long)k * a.gridx] = acc64[k] + (double)acc[k];
+    for (int m = 0; m < 2; ++m) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) half[i] = acc[32 * m + i];
+      const double s = warp_transpose_sum(half, lane);
+      L.partial[(long long)grp * L.n_ent + (sub.tile0 + warp) * 64 + 32 * m + lane] = s;
+    }
   }
 }
 
-// msum[map[tile][k]] = scale * sum over blocks of partial[tile][k][block], in a fixed order
-// (added to msum when accumulating x-slabs).
-// One warp per (tile, entry): lane l adds the block sums b = l, l + 32, ... (contiguous loads
-// across the warp), then the lanes' sums are added by a fixed shuffle tree.
-__global__ void reduce_partials_kernel(ContractArgs a) {
-  const int idx = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (idx >= a.ntiles * 16) return;  // warp-uniform
-  const int dst = a.tile_map[idx];
-  if (dst < 0) return;  // warp-uniform
-  const double* src = a.partial + (long long)idx * a.gridx;
+// ---------------------------------------------------------------- FP64
+// Warp = (level, set of kSumJobs jobs, run of spw steps of 32 voxels), lane = voxel.
+__global__ void __launch_bounds__(32 * kF64Warps, 4) contract_f64_kernel(SumArgs a) {
+  __shared__ long long foff[kF64Warps][kSumJobs][6];
+  __shared__ int fcnt[kF64Warps][kSumJobs];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = blockIdx.x * kF64Warps + warp;
+  if (w >= a.items) return;  // warp-uniform; no block barrier below
+  const SumLevel L = level_of(a, w);
+  const int unit = w - L.w0;
+  const int split = unit / L.units, set = unit - split * L.units;
+  const double* fields = static_cast<const double*>(a.fields);
+  if (lane < kSumJobs) {
+    const int j = set * kSumJobs + lane;
+    SumJob job{};
+    if (j < L.njobs) job = L.jobs[j];
+    fcnt[warp][lane] = job.n;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) foff[warp][lane][i] = (long long)job.f[i] * L.fstride;
+  }
+  __syncwarp();
+  // Sums of kF64Run steps are added over the warp before they join the total: a lane that meets the
+  // counting fields' peak at the origin would otherwise round every later addition at its size.
+  double total = 0.0;
+  const long long v0 = (long long)split * L.spw * 32;
+  for (int k0 = 0; k0 < L.spw; k0 += kF64Run) {
+    double acc[4 * kSumJobs];
+#pragma unroll
+    for (int i = 0; i < 4 * kSumJobs; ++i) acc[i] = 0.0;
+    const int k1 = min(k0 + kF64Run, L.spw);
+    for (int k = k0; k < k1; ++k) {
+      const long long v = v0 + 32LL * k + lane;
+      const bool in = v < L.nvox;
+      long long o = in ? v : 0;
+      if (L.t > 1 && in) {
+        const unsigned g = (unsigned)L.g, u = (unsigned)v;
+        const unsigned xy = u / g, z = u - xy * g, x = xy / g, y = xy - x * g;
+        o = ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
+      }
+      if (!in) continue;  // the ragged end: the lane adds nothing
+      const double* f = fields + o;
+#pragma unroll
+      for (int j = 0; j < kSumJobs; ++j) {
+        const int n = fcnt[warp][j];  // warp-uniform
+        if (n == 0) break;
+        const long long* fo = foff[warp][j];
+        const double p = f[fo[0]] * f[fo[1]];
+        const double d0 = f[fo[2]], d1 = f[fo[3]], d2 = f[fo[4]], d3 = f[fo[5]];
+        acc[4 * j] = fma(p, d0, acc[4 * j]);
+        if (n > 1) acc[4 * j + 1] = fma(p, d1, acc[4 * j + 1]);
+        if (n > 2) acc[4 * j + 2] = fma(p, d2, acc[4 * j + 2]);
+        if (n > 3) acc[4 * j + 3] = fma(p, d3, acc[4 * j + 3]);
+      }
+    }
+    total += warp_transpose_sum(acc, lane);
+  }
+  const int e = set * 4 * kSumJobs + lane;
+  if (e < L.n_ent) L.partial[(long long)split * L.n_ent + e] = total;
+}
+
+// msum[map[e]] = scale * sum over the splits of partial[.][e] (added to msum when accumulating
+// x-slabs). A block takes 8 neighbouring outputs, 32 threads each: thread (e, k) adds splits k,
+// k + 32, ..., then the 32 sums are added in order. (A warp of outputs a block, 8 threads each, left
+// small plans with 5 blocks of long dependent chains: 18.5 us of an Ng = 32 FP64 estimate.)
+constexpr int kReduceOuts = 8;
+__global__ void __launch_bounds__(256) reduce_sums_kernel(SumArgs a) {
+  __shared__ double part[32][kReduceOuts + 1];
+  const int o = threadIdx.x % kReduceOuts, k = threadIdx.x / kReduceOuts;
+  const int idx = blockIdx.x * kReduceOuts + o;
+  int l = 0;
+  while (l + 1 < a.n_lv && idx >= a.lv[l + 1].ent0) ++l;
+  const SumLevel L = a.lv[l];
+  const int e = idx - L.ent0;
+  const int dst = idx < a.n_ent ? L.map[e] : -1;
   double s = 0.0;
-  for (int b = lane; b < a.gridx; b += 32) s += src[b];
+  if (dst >= 0) {
+#pragma unroll 4
+    for (int b = k; b < L.splits; b += 32) s += L.partial[(long long)b * L.n_ent + e];
+  }
+  part[k][o] = s;
+  __syncthreads();
+  if (k == 0 && dst >= 0) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  if (lane == 0) a.msum[dst] = a.accumulate ? a.msum[dst] + a.scale * s : a.scale * s;
+    for (int w = 1; w < 32; ++w) s += part[w][o];
+    a.msum[dst] = a.accumulate ? a.msum[dst] + L.scale * s : L.scale * s;
+  }
 }
 
-template <typename T>
-bsp_status launch_contract_simt(const ContractArgs& a, cudaStream_t s) {
-  if (a.ntiles == 0) return BSP_OK;
-  const long long chunks = (a.nvox + kChunk - 1) / kChunk;
-  const long long per_block_chunks = (chunks + a.gridx - 1) / a.gridx;
-  const long long vpb = per_block_chunks * kChunk;
-  dim3 grid(a.gridx, (a.ntiles + kContractThreads - 1) / kContractThreads);
-  const size_t smem = 2 * (size_t)a.ns * kChunkLd * sizeof(T);
-  BSP_CUDA(cudaFuncSetAttribute(contract_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem));
-  contract_simt_kernel<T><<<grid, kContractThreads, smem, s>>>(a, vpb);
+}  // namespace
+
+template <>
+bsp_status launch_contract_simt<float>(const SumArgs& a, cudaStream_t s) {
+  if (a.items == 0) return BSP_OK;
+  BSP_CUDA(cudaFuncSetAttribute(contract_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem));
+  contract_f32_kernel<<<a.items, kSumThreads, a.smem, s>>>(a);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;
 }
 
-bsp_status launch_reduce_partials(const ContractArgs& a, cudaStream_t s) {
-  const long long n = (long long)a.ntiles * 16 * 32;  // one warp per entry
-  if (n == 0) return BSP_OK;
-  reduce_partials_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a);
+template <>
+bsp_status launch_contract_simt<double>(const SumArgs& a, cudaStream_t s) {
+  if (a.items == 0) return BSP_OK;
+  contract_f64_kernel<<<(a.items + kF64Warps - 1) / kF64Warps, 32 * kF64Warps, 0, s>>>(a);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;
 }
+
+bsp_status launch_reduce_sums(const SumArgs& a, cudaStream_t s) {
+  if (a.n_ent == 0) return BSP_OK;
+  reduce_sums_kernel<<<(a.n_ent + kReduceOuts - 1) / kReduceOuts, 32 * kReduceOuts, 0, s>>>(a);
+  BSP_CUDA(cudaGetLastError());
+  return BSP_OK;
+}
+
+int sum_stage_bytes(int nf) { return 2 * nf * kSumFieldBytes; }
 
 // ---------------------------------------------------------------- product fields (order 4)
 template <typename T>
@@ -193,15 +409,12 @@ bsp_status launch_pair_fields(const void* f, long long nvox, const int2* pairs, 
 
 template bsp_status launch_pair_fields<float>(const void*, long long, const int2*, int, void*, int, cudaStream_t);
 template bsp_status launch_pair_fields<double>(const void*, long long, const int2*, int, void*, int, cudaStream_t);
-template bsp_status launch_contract_simt<float>(const ContractArgs&, cudaStream_t);
-template bsp_status launch_contract_simt<double>(const ContractArgs&, cudaStream_t);
 
 // ---------------------------------------------------------------- level fields
-// dst[j][x][y][z] = src[shells[j]][t x][t y][t z]: the fields of a coarser level sampled from the
-// evaluation grid (side S) with stride t.
-template <typename T>
-__global__ void decimate_kernel(const T* __restrict__ src, int S, const int* __restrict__ shells, int nsh,
-                                T* __restrict__ dst, int g, int t) {
+// dst[j][x][y][z] = src[shells[j]][t x][t y][t z]: the split fields of a coarser level sampled from
+// the evaluation grid (side S) with stride t.
+__global__ void decimate_kernel(const uint16_t* __restrict__ src, int S, const int* __restrict__ shells, int nsh,
+                                uint16_t* __restrict__ dst, int g, int t) {
   const long long per = (long long)g * g * g;
   const long long total = per * nsh;
   const long long plane = (long long)S * S;
@@ -216,20 +429,15 @@ __global__ void decimate_kernel(const T* __restrict__ src, int S, const int* __r
   }
 }
 
-template <typename T>
-bsp_status launch_decimate(const void* src, int S, const int* shells, int nsh, void* dst, int g, int t, int n_sm,
-                           cudaStream_t s) {
+bsp_status launch_decimate(const uint16_t* src, int S, const int* shells, int nsh, uint16_t* dst, int g, int t,
+                           int n_sm, cudaStream_t s) {
   const long long total = (long long)g * g * g * nsh;
   if (total == 0) return BSP_OK;
   long long blocks = std::min<long long>((total + 255) / 256, 16LL * n_sm);
-  decimate_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const T*>(src), S, shells, nsh, static_cast<T*>(dst),
-                                                     g, t);
+  decimate_kernel<<<(unsigned)blocks, 256, 0, s>>>(src, S, shells, nsh, dst, g, t);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;
 }
-template bsp_status launch_decimate<float>(const void*, int, const int*, int, void*, int, int, int, cudaStream_t);
-template bsp_status launch_decimate<double>(const void*, int, const int*, int, void*, int, int, int, cudaStream_t);
-template bsp_status launch_decimate<uint16_t>(const void*, int, const int*, int, void*, int, int, int, cudaStream_t);
 
 // ---------------------------------------------------------------- finalize
 // b_trip[t] = norm msum[t] / tsum[t]                     (Eq. (2.7) with Eq. (2.10))

@@ -4,6 +4,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -101,37 +103,240 @@ void make_items(const bsp_plan* p, const PassLines& lines, std::vector<Item>& xi
   make_items_g(p->geom, p->ngs, lines, xi, yi, zi);
 }
 
-// Tiles of up to 4 consecutive pairs x 4 consecutive c over a list of bins sorted by (a, b, c).
-void make_tiles(const std::vector<int>& ta, const std::vector<int>& tb, const std::vector<int>& tc,
-                std::vector<int2>& pairs, std::vector<Tile>& tiles, std::vector<int>& map,
-                const std::vector<int>* ids) {
-  pairs.clear(); tiles.clear(); map.clear();
-  std::vector<std::vector<std::pair<int, int>>> pc;  // per pair: (c, bin)
+// 4 x 4 tiles of 4 consecutive pairs and 4 aligned c that hold a bin of a list sorted by (a, b, c):
+// the measure the number of summation blocks follows (see divide_sum_level).
+static int count_pair_quads(const std::vector<int>& ta, const std::vector<int>& tb, const std::vector<int>& tc) {
+  int n = 0, pair = -1;
+  std::vector<int> quads;  // of the current 4 pairs
+  auto close = [&]() {
+    std::sort(quads.begin(), quads.end());
+    n += (int)(std::unique(quads.begin(), quads.end()) - quads.begin());
+    quads.clear();
+  };
   for (size_t t = 0; t < ta.size(); ++t) {
-    if (pairs.empty() || pairs.back().x != ta[t] || pairs.back().y != tb[t]) {
-      pairs.push_back(make_int2(ta[t], tb[t]));
-      pc.emplace_back();
+    if (t == 0 || ta[t] != ta[t - 1] || tb[t] != tb[t - 1]) {
+      ++pair;
+      if (pair % 4 == 0) close();
     }
-    pc.back().push_back({tc[t], ids ? (*ids)[t] : (int)t});
+    quads.push_back(tc[t] / 4);
   }
-  const int np = (int)pairs.size();
-  for (int p0 = 0; p0 < np; p0 += 4) {
-    const int cnt = std::min(4, np - p0);
-    int cmin = 1 << 30, cmax = -1;
-    for (int i = 0; i < cnt; ++i)
-      for (auto& e : pc[p0 + i]) { cmin = std::min(cmin, e.first); cmax = std::max(cmax, e.first); }
-    for (int c0 = cmin - cmin % 4; c0 <= cmax; c0 += 4) {
-      int m[16];
-      bool any = false;
-      for (int k = 0; k < 16; ++k) m[k] = -1;
-      for (int i = 0; i < cnt; ++i)
-        for (auto& e : pc[p0 + i])
-          if (e.first >= c0 && e.first < c0 + 4) { m[i * 4 + (e.first - c0)] = e.second; any = true; }
-      if (!any) continue;
-      tiles.push_back({p0, cnt, c0, 0});
-      for (int k = 0; k < 16; ++k) map.push_back(m[k]);
+  close();
+  return n;
+}
+
+// FP32 tables of a CUDA-core contraction level: tiles of 2 a x 4 (2) b x 8 (4) c taken off the bins from
+// the largest shells down, then blocks of `per` tiles of one kind that share fields, with the
+// fields they read. out[64 t + 32 i + 8 j + k]: the bin of output (i, j, k) of tile t.
+struct SumRaw { int a[2], b[4], c[8], kind, out[64]; };
+static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std::vector<int>& tb,
+                                          const std::vector<int>& tc, const std::vector<int>* ids, int ncmax) {
+  std::vector<SumRaw> raw;
+  struct B { int a, b, c, id; };
+  std::vector<B> bins;
+  for (size_t t = 0; t < ta.size(); ++t) bins.push_back({ta[t], tb[t], tc[t], ids ? (*ids)[t] : (int)t});
+  auto distinct = [](std::vector<int> v) {  // descending
+    std::sort(v.begin(), v.end(), std::greater<int>());
+    v.erase(std::unique(v.begin(), v.end()), v.end());
+    return v;
+  };
+  const std::vector<int> as = distinct(ta);
+  for (size_t i = 0; i < as.size(); i += 2) {
+    const int na = (int)std::min<size_t>(2, as.size() - i);
+    std::vector<B> sel;
+    std::vector<int> bs;
+    for (const B& x : bins)
+      if (x.a == as[i] || (na > 1 && x.a == as[i + 1])) { sel.push_back(x); bs.push_back(x.b); }
+    bs = distinct(bs);
+    for (size_t j = 0, nb; j < bs.size(); j += nb) {
+      nb = std::min<size_t>(bs.size() - j, 4);
+      std::vector<B> rows;
+      std::vector<int> cs;
+      for (const B& x : sel)
+        for (size_t k = 0; k < nb; ++k)
+          if (x.b == bs[j + k]) { rows.push_back(x); cs.push_back(x.c); }
+      std::sort(cs.begin(), cs.end());
+      cs.erase(std::unique(cs.begin(), cs.end()), cs.end());
+      for (size_t m = 0, nc; m < cs.size(); m += nc) {
+        nc = std::min<size_t>(cs.size() - m, ncmax);
+        SumRaw t;
+        std::vector<int> ub;  // the b with a bin here
+        for (size_t k = 0; k < nb; ++k)
+          for (const B& x : rows)
+            if (x.b == bs[j + k] && x.c >= cs[m] && x.c <= cs[m + nc - 1]) { ub.push_back(x.b); break; }
+        // places without a shell repeat the first
+        for (int k = 0; k < 2; ++k) t.a[k] = as[i + (k < na ? k : 0)];
+        for (size_t k = 0; k < 4; ++k) t.b[k] = ub[k < ub.size() ? k : 0];
+        for (size_t k = 0; k < 8; ++k) t.c[k] = cs[m + (k < nc ? k : 0)];
+        t.kind = (ub.size() > 2 ? 2 : 0) + (nc > 4 ? 1 : 0);
+        for (int& o : t.out) o = -1;
+        for (const B& x : rows)
+          for (int ia = 0; ia < na; ++ia)
+            for (size_t ib = 0; ib < ub.size(); ++ib)
+              for (size_t ic = 0; ic < nc; ++ic)
+                if (x.a == t.a[ia] && x.b == t.b[ib] && x.c == t.c[ic]) t.out[32 * ia + 8 * ib + ic] = x.id;
+        raw.push_back(t);
+      }
     }
   }
+  std::stable_sort(raw.begin(), raw.end(), [](const SumRaw& x, const SumRaw& y) { return x.kind > y.kind; });
+  return raw;
+}
+
+static void make_sum_subs(std::vector<SumRaw> raw, int per, std::vector<SumTile>& tiles, std::vector<SumSub>& subs,
+                          std::vector<int>& sub_fields, std::vector<int>& map) {
+  while (!raw.empty()) {  // the first tile left, then those of its kind that add the fewest fields
+    SumSub sub{(int)tiles.size(), 0, (int)sub_fields.size(), 0, raw.front().kind};
+    std::vector<int> cur;
+    auto with = [&](const SumRaw& t) {
+      std::vector<int> u = cur;
+      auto add = [&](const int* f, int n) {
+        for (int k = 0; k < n; ++k)
+          if (std::find(u.begin(), u.end(), f[k]) == u.end()) u.push_back(f[k]);
+      };
+      add(t.a, 2);
+      add(t.b, 4);
+      add(t.c, 8);
+      return u;
+    };
+    while (sub.ntiles < per && !raw.empty()) {
+      size_t best = 0, best_n = (size_t)-1;
+      for (size_t k = 0; k < raw.size() && raw[k].kind == sub.kind; ++k) {
+        const size_t n = with(raw[k]).size();
+        if (n < best_n) { best = k; best_n = n; }
+        if (cur.empty()) break;
+      }
+      if (best_n == (size_t)-1 || (!cur.empty() && best_n > (size_t)kSumMaxFields)) break;
+      const SumRaw t = raw[best];
+      raw.erase(raw.begin() + (long)best);
+      cur = with(t);
+      SumTile s{};
+      auto at = [&](int f) { return (uint8_t)(std::find(cur.begin(), cur.end(), f) - cur.begin()); };
+      for (int k = 0; k < 2; ++k) s.a[k] = at(t.a[k]);
+      for (int k = 0; k < 4; ++k) s.b[k] = at(t.b[k]);
+      for (int k = 0; k < 8; ++k) s.c[k] = at(t.c[k]);
+      tiles.push_back(s);
+      map.insert(map.end(), t.out, t.out + 64);
+      sub.ntiles += 1;
+    }
+    sub.nf = (int)cur.size();
+    sub_fields.insert(sub_fields.end(), cur.begin(), cur.end());
+    subs.push_back(sub);
+  }
+}
+
+// FP64 jobs of a CUDA-core contraction level: each pair's third shells four at a time.
+static void make_sum_jobs(const std::vector<int>& ta, const std::vector<int>& tb, const std::vector<int>& tc,
+                          const std::vector<int>* ids, std::vector<SumJob>& jobs, std::vector<int>& map) {
+  for (size_t t = 0; t < ta.size(); ++t) {
+    if (t == 0 || ta[t] != ta[t - 1] || tb[t] != tb[t - 1] || jobs.back().n == 4) {
+      jobs.push_back({{ta[t], tb[t], tc[t], tc[t], tc[t], tc[t]}, 0, 0});
+      map.insert(map.end(), 4, -1);
+    }
+    SumJob& j = jobs.back();
+    for (int k = j.n; k < 4; ++k) j.f[2 + k] = tc[t];
+    map[map.size() - 4 + j.n] = ids ? (*ids)[t] : (int)t;
+    j.n += 1;
+  }
+}
+
+// FP32: the summation blocks of `nvox` voxels (a multiple of 64 voxels each), their whole runs in
+// groups of kSumRuns and their remainders likewise. FP64: steps of 32 voxels, spw of them per warp.
+static void divide_sum_level(SumLevel* l, long long nvox, int spw, bool f64) {
+  l->nvox = nvox;
+  if (f64) {
+    l->spw = spw;
+    l->splits = (int)((nvox + 32LL * spw - 1) / (32LL * spw));
+    return;
+  }
+  const long long chunks = (nvox + 63) / 64;
+  l->vpb = (int)((chunks + l->nblk_cap - 1) / l->nblk_cap * 64);
+  l->nblk = (int)((nvox + l->vpb - 1) / l->vpb);
+  l->nfull = l->vpb / kSumRun;
+  l->ngf = (int)(((long long)l->nblk * l->nfull + kSumRuns - 1) / kSumRuns);
+  l->splits = l->ngf + (l->vpb % kSumRun ? (l->nblk + kSumRuns - 1) / kSumRuns : 0);
+}
+
+bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::vector<int>& tb,
+                          const std::vector<int>& tc, const std::vector<int>* ids, bool f64, long long nvox,
+                          SumLevel* lev, std::vector<void*>* owned, cudaStream_t s) {
+  SumLevel& l = *lev;
+  bsp_status st = BSP_OK;
+  auto up = [&](const auto& v, auto** d) {
+    st = dev_upload(p, v, d, s);
+    if (st == BSP_OK && owned) owned->push_back(*d);
+    return st;
+  };
+  std::vector<int> map;
+  if (f64) {
+    std::vector<SumJob> jobs;
+    make_sum_jobs(ta, tb, tc, ids, jobs, map);
+    SumJob* dj = nullptr;
+    if (up(jobs, &dj) != BSP_OK) return st;
+    l.jobs = dj;
+    l.njobs = (int)jobs.size();
+    l.units = (l.njobs + kSumJobs - 1) / kSumJobs;
+  } else {
+    // FP32 runs start at the summation blocks' first voxels: 4 blocks per SM, divided by the blocks
+    // of 256 4 x 4 tiles
+    const int gy = std::max((count_pair_quads(ta, tb, tc) + 255) / 256, 1);
+    l.nblk_cap = (int)std::min<long long>(std::max(4 * p->n_sm / gy, 1), (nvox + 63) / 64);
+    divide_sum_level(&l, nvox, 1, false);
+    // 8 c a tile; 4 (more tiles, each about half as long) on levels too small to give every SM 8;
+    // then as many tiles a block as give every SM one
+    std::vector<SumRaw> raw = make_sum_tiles(ta, tb, tc, ids, 8);
+    if ((long long)raw.size() * l.splits < (long long)kSumWarps * p->n_sm) raw = make_sum_tiles(ta, tb, tc, ids, 4);
+    const long long each = ((long long)raw.size() * l.splits + p->n_sm - 1) / p->n_sm;
+    const int per = (int)std::max<long long>(1, std::min<long long>(kSumWarps, each));
+    std::vector<SumTile> tiles;
+    std::vector<SumSub> subs;
+    std::vector<int> fields;
+    make_sum_subs(std::move(raw), per, tiles, subs, fields, map);
+    SumTile* dt = nullptr;
+    SumSub* ds = nullptr;
+    int* df = nullptr;
+    if (up(tiles, &dt) != BSP_OK || up(subs, &ds) != BSP_OK || up(fields, &df) != BSP_OK) return st;
+    l.tiles = dt;
+    l.subs = ds;
+    l.sub_fields = df;
+    l.units = (int)subs.size();
+    for (const SumSub& x : subs) l.max_nf = std::max(l.max_nf, x.nf);
+  }
+  int* dm = nullptr;
+  if (up(map, &dm) != BSP_OK) return st;
+  l.map = dm;
+  l.n_ent = (int)map.size();
+  return BSP_OK;
+}
+
+bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel> lv, const std::vector<long long>& nvox, int spw, bool f64,
+                         SumArgs* out, std::vector<void*>* owned, cudaStream_t s) {
+  SumArgs a{};
+  bsp_status st;
+  for (size_t i = 0; i < lv.size(); ++i) {
+    SumLevel& l = lv[i];
+    divide_sum_level(&l, nvox[i], spw, f64);
+    l.w0 = a.items;
+    l.ent0 = a.n_ent;
+    a.items += l.units * l.splits;
+    a.n_ent += l.n_ent;
+    if (!f64) a.smem = std::max(a.smem, sum_stage_bytes(l.max_nf));
+    void* d = nullptr;
+    if ((st = dev_alloc(p, (size_t)l.splits * l.n_ent * sizeof(double), &d)) != BSP_OK) return st;
+    if (owned) owned->push_back(d);
+    l.partial = static_cast<double*>(d);
+  }
+  SumLevel* d = nullptr;
+  if ((st = dev_upload(p, lv, &d, s)) != BSP_OK) return st;
+  if (owned) owned->push_back(d);
+  a.lv = d;
+  a.n_lv = (int)lv.size();
+  *out = a;
+  return BSP_OK;
+}
+
+// FP64 steps per warp for `steps` (job set, 32 voxels) steps in a launch: about 48 warps per SM.
+static int sum_steps_per_warp(long long steps, int n_sm) {
+  return (int)std::max<long long>(1, (steps + 48LL * n_sm - 1) / (48LL * n_sm));
 }
 
 // Pair groups of the tensor-core contraction (see TcArgs). A slot holds three fields f0, f1, f2
@@ -381,17 +586,6 @@ bsp_status run_passes(const bsp_plan* p, const void* spec, int rsd, void* tw, vo
   a.slab_nx = slab_nx;
   return launch_zpass<T>(a, nzi, lines.z, s);
 }
-
-int pick_gridx_n(int n_sm, int ntiles, long long nvox) {
-  const int gy = (ntiles + 255) / 256;
-  int gx = (4 * n_sm) / std::max(gy, 1);
-  gx = std::max(gx, 1);
-  const long long chunks = (nvox + 63) / 64;
-  if (gx > chunks) gx = (int)chunks;
-  return gx;
-}
-
-int pick_gridx(const bsp_plan* p, int ntiles) { return pick_gridx_n(p->n_sm, ntiles, p->nvox()); }
 
 bsp_status validate(const bsp_plan_desc* d) {
   if (!d) return fail(BSP_ERR_INVALID_ARG, "desc is NULL");
@@ -758,6 +952,47 @@ void merge_tc_levels(const bsp_plan* p, std::vector<std::pair<int, std::vector<i
   }
 }
 
+// The CUDA-core contraction launches of the plan: every level at once, largest first; a plan
+// streaming x-slabs has one level and two slab lengths.
+bsp_status build_sums(bsp_plan* p, cudaStream_t s) {
+  const bool f64 = p->prec == BSP_FP64;
+  const int last = p->n_slabs() - 1;
+  std::vector<SumLevel> lv;
+  std::vector<long long> nvox[2];
+  bsp_status st;
+  for (size_t i = p->levels.size(); i-- > 0;) {
+    const ContractLevel& L = p->levels[i];
+    std::vector<int> ta, tb, tc;
+    for (int b : L.bins) {
+      const bsp_triplet& t = p->trips[b];
+      ta.push_back(t.a);
+      tb.push_back(t.b);
+      tc.push_back(p->order == 4 ? p->ns + p->pid4(t.c, t.e) : t.c);
+    }
+    SumLevel l{};
+    l.g = L.g;
+    l.t = L.stride;
+    l.s = p->ngs;
+    l.scale = L.scale;
+    const long long n0 = p->slab_nx ? (long long)p->slab_len(0) * p->ngs * p->ngs : L.nvox();
+    const long long n1 = p->slab_nx ? (long long)p->slab_len(last) * p->ngs * p->ngs : n0;
+    st = make_sum_level(p, ta, tb, tc, &L.bins, f64, p->slab_nx ? p->nvox() : n0, &l, nullptr, s);
+    if (st != BSP_OK) return st;
+    lv.push_back(l);
+    nvox[0].push_back(n0);
+    nvox[1].push_back(n1);
+  }
+  long long steps = 0;
+  for (size_t i = 0; i < lv.size(); ++i) steps += (nvox[0][i] + 31) / 32 * lv[i].units;
+  const int spw = sum_steps_per_warp(steps, p->n_sm);
+  for (int k = 0; k < 2; ++k) {
+    for (size_t i = 0; i < lv.size(); ++i) lv[i].fstride = p->slab_nx ? nvox[k][i] : p->nvox();
+    if (k == 1 && nvox[1] == nvox[0]) p->sums_last = p->sums;
+    else if ((st = make_sum_args(p, lv, nvox[k], spw, f64, k ? &p->sums_last : &p->sums, nullptr, s)) != BSP_OK) return st;
+  }
+  return BSP_OK;
+}
+
 // Contraction levels (see ContractLevel): each pair (a, b) of the kept bins goes to the smallest
 // divisor g of the evaluation grid (g % 8 == 0, g >= 16) above r_a + r_b + r_cmax - 3, the largest
 // wavevector component of its triple products; split-BF16 plans then merge levels where the
@@ -814,19 +1049,18 @@ bsp_status build_levels(bsp_plan* p, cudaStream_t s) {
         if (used[n]) { loc[n] = (int)L.shells.size(); L.shells.push_back(n); }
     }
     const int nsh = (int)L.shells.size();
-    std::vector<int> la, lb, lc;
-    for (int b : L.bins) {
-      const bsp_triplet& t = p->trips[b];
-      la.push_back(loc[t.a]);
-      lb.push_back(loc[t.b]);
-      lc.push_back(p->order == 4 ? p->ns + p->pid4(t.c, t.e) : loc[t.c]);  // order 4: top level only
-    }
-    std::vector<int2> pairs;
-    std::vector<Tile> tiles;
-    std::vector<int> map;
-    make_tiles(la, lb, lc, pairs, tiles, map, &L.bins);
     void* tmp = nullptr;
     if (p->prec == BSP_MIXED_BF16X3) {
+      std::vector<int> la, lb, lc;
+      for (int b : L.bins) {
+        const bsp_triplet& t = p->trips[b];
+        la.push_back(loc[t.a]);
+        lb.push_back(loc[t.b]);
+        lc.push_back(loc[t.c]);
+      }
+      std::vector<int2> pairs;
+      for (size_t i = 0; i < la.size(); ++i)
+        if (i == 0 || la[i] != la[i - 1] || lb[i] != lb[i - 1]) pairs.push_back(make_int2(la[i], lb[i]));
       L.np = tc_padded_shells(nsh);
       const TcGrouping G = group_pairs(pairs, nsh, L.np == 32 ? 3 : 2);
       L.kt = G.kt;
@@ -854,20 +1088,10 @@ bsp_status build_levels(bsp_plan* p, cudaStream_t s) {
       if ((st = dev_alloc(p, tc_partial_entries(std::max(L.n_tg, 1), std::max(L.kt, 1), std::max(L.gridy, L.gridy_cap), L.np) * sizeof(float2), &tmp)) != BSP_OK)
         return st;
       L.tc_partial = static_cast<float2*>(tmp);
-    } else {
-      L.ntiles = (int)tiles.size();
-      L.gridx = pick_gridx_n(p->n_sm, L.ntiles, L.nvox());
-      if ((st = dev_upload(p, tiles, &L.d_tiles, s)) != BSP_OK) return st;
-      if ((st = dev_upload(p, pairs, &L.d_pairs, s)) != BSP_OK) return st;
-      if ((st = dev_upload(p, map, &L.d_map, s)) != BSP_OK) return st;
-      if ((st = dev_alloc(p, (size_t)std::max(L.gridx, 1) * std::max(L.ntiles, 1) * 16 * sizeof(double), &tmp)) != BSP_OK)
-        return st;
-      L.partial = static_cast<double*>(tmp);
     }
-    if (!L.top) {
-      std::vector<int> src = L.shells;
-      if (p->prec == BSP_MIXED_BF16X3)  // split planes: high parts, then low parts (ns planes later)
-        for (int n : L.shells) src.push_back(p->ns + n);
+    if (!L.top && p->prec == BSP_MIXED_BF16X3) {
+      std::vector<int> src = L.shells;  // split planes: high parts, then low parts (ns planes later)
+      for (int n : L.shells) src.push_back(p->ns + n);
       if ((st = dev_upload(p, src, &L.d_shells, s)) != BSP_OK) return st;
       if ((st = dev_alloc(p, (size_t)nsh * (size_t)L.nvox() * re, &L.fields)) != BSP_OK) return st;
     }
@@ -898,6 +1122,9 @@ bsp_status build_levels(bsp_plan* p, cudaStream_t s) {
   }
   if (p->prec == BSP_MIXED_BF16X3 && p->autotune && !p->slab_nx) {
     if ((st = autotune_levels(p, s)) != BSP_OK) return st;
+  }
+  if (p->prec != BSP_MIXED_BF16X3) {
+    if ((st = build_sums(p, s)) != BSP_OK) return st;
   }
   if (p->prec == BSP_MIXED_BF16X3) {
     std::vector<TcBin> tb(p->trips.size());
@@ -980,44 +1207,36 @@ bsp_status plan_sums(bsp_plan* p, bool lengths, const std::vector<int>& ca, cons
     if (lengths)
       TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, f, dxi, (int)xi.size(), dyi, (int)yi.size(), dzi, 0, lines, s, 1, true, false));
   }
-  std::vector<int2> pairs;
-  std::vector<Tile> tiles;
-  std::vector<int> map;
-  make_tiles(ca, cb, cc, pairs, tiles, map, ids);
-  Tile* dt = nullptr; int2* dp = nullptr; int* dm = nullptr;
-  TRY(dev_upload(p, tiles, &dt, s)); tmp.push_back(dt);
-  TRY(dev_upload(p, pairs, &dp, s)); tmp.push_back(dp);
-  TRY(dev_upload(p, map, &dm, s)); tmp.push_back(dm);
-  ContractArgs c{};
-  c.fields = f;
-  c.nvox = slab_vox;
-  c.ns = nf;
-  c.tiles = dt;
-  c.pairs = dp;
-  c.tile_map = dm;
-  c.ntiles = (int)tiles.size();
-  c.gridx = pick_gridx_n(p->n_sm, c.ntiles, slab_vox);
-  void* part = nullptr; void* ms = nullptr;
-  TRY(dev_alloc(p, (size_t)c.gridx * c.ntiles * 16 * sizeof(double), &part)); tmp.push_back(part);
+  std::vector<SumLevel> lv(1);
+  lv[0].t = 1;
+  lv[0].scale = 1.0;  // scaled to the ng^3 grid on the host
+  TRY(make_sum_level(p, ca, cb, cc, ids, true, slab_vox, &lv[0], &tmp, s));
+  const int spw = sum_steps_per_warp((slab_vox + 31) / 32 * lv[0].units, p->n_sm);
+  void* ms = nullptr;
   TRY(dev_alloc(p, ca.size() * sizeof(double), &ms)); tmp.push_back(ms);
-  c.partial = static_cast<double*>(part);
-  c.msum = static_cast<double*>(ms);
-  c.n_out = (int)ca.size();
-  c.scale = 1.0;  // scaled to the ng^3 grid on the host
+  SumArgs sums[2];  // a full slab's (or the grid's), the last slab's
+  for (int k = 0; k < 2; ++k) {
+    const int len = k && slab ? S - (nsl - 1) * nx : nx;
+    lv[0].fstride = p->dim == 2 ? slab_vox : (long long)len * S * S;
+    if (k && (!slab || len == nx)) { sums[1] = sums[0]; continue; }
+    TRY(make_sum_args(p, lv, {lv[0].fstride}, spw, true, &sums[k], &tmp, s));
+  }
   for (int k = 0; k < nsl; ++k) {
     if (slab) {  // the slab's fields, [nf][x - x0][y][z]
       const int x0 = k * nx, len = std::min(nx, S - x0);
       const int nzk = zoff[k + 1] - zoff[k];
-      c.nvox = (long long)len * S * S;
       TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2, f, dxi, 0, dyi, 0, dzi + zoff[k], nzk, lines, s, 0, false,
                              true, x0, len));
       if (lengths)
-        TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, static_cast<double*>(f) + (size_t)p->ns * c.nvox, dxi, 0,
-                               dyi, 0, dzi + zoff[k], nzk, lines, s, 1, false, true, x0, len));
+        TRY(run_passes<double>(p, nullptr, 0, tw, g1, g2w, static_cast<double*>(f) + (size_t)p->ns * ((size_t)len * S * S),
+                               dxi, 0, dyi, 0, dzi + zoff[k], nzk, lines, s, 1, false, true, x0, len));
     }
+    SumArgs c = sums[k == nsl - 1];
+    c.fields = f;
+    c.msum = static_cast<double*>(ms);
     c.accumulate = k > 0;
     TRY(launch_contract_simt<double>(c, s));
-    TRY(launch_reduce_partials(c, s));
+    TRY(launch_reduce_sums(c, s));
   }
   tsum.assign(ca.size(), 0.0);
   cudaError_t e = cudaMemcpyAsync(tsum.data(), ms, ca.size() * sizeof(double), cudaMemcpyDeviceToHost, s);

@@ -114,10 +114,53 @@ bsp_status launch_warp_zfpass(const PassArgs& a, const float* gfield, long long 
 bsp_status launch_warp_yfpass(const PassArgs& a, int n_items, cudaStream_t s);
 bsp_status launch_warp_xfpass(const PassArgs& a, int n_items, float scale, cudaStream_t s);
 
-// ---------------------------------------------------------------- contraction tables
-// A tile covers up to 4 consecutive pairs and 4 consecutive c shells; map[16] gives the kept
-// bin of output (i, j) or -1.
-struct Tile { int p0, np, c0, pad; };
+// ---------------------------------------------------------------- CUDA-core contraction tables
+// FP32: a tile is 2 x (4 or 2) x (8 or 4) outputs (a, b, c), one warp's registers; a sub is the up to
+// kSumWarps tiles of one block, of one kind (2 [4 b] + [8 c]), and the fields it stages; tiles name
+// fields by their place in that list. FP64: a job is one pair and n <= 4 third fields: f = (a, b, c0
+// .. c3).
+struct SumTile { uint8_t a[2], b[4], c[8], pad[2]; };
+struct SumSub { int tile0, ntiles, field0, nf, kind; };
+struct SumJob { int f[6], n, pad; };
+
+constexpr int kSumWarps = 8;      // warps (tiles) of an FP32 block
+constexpr int kSumMaxFields = 27; // fields an FP32 block stages at most (a tile has up to 14)
+constexpr int kSumRuns = 32;      // runs of an FP32 block, one per lane
+constexpr int kSumRun = 1024;     // voxels of one FP32 accumulation run
+constexpr int kSumJobs = 8;       // FP64 jobs of a warp
+
+// One level of a CUDA-core contraction launch: triple sums over the g^3 voxels sampled from source
+// fields of side s with stride t (t == 1: over the nvox voxels as they lie in memory). Its work
+// items, numbered from w0 on, are FP32 blocks (a sub, a group of kSumRuns runs) or FP64 warps (a set
+// of kSumJobs jobs, spw steps of 32 voxels); each writes one partial sum of its outputs.
+struct SumLevel {
+  long long nvox;          // voxels summed by this call
+  long long fstride;       // elements between source fields
+  int g, t, s;
+  int w0, units, splits;   // first item; items = units (subs or job sets) x splits
+  int nblk_cap, nblk, vpb; // FP32: summation blocks (at most, now), voxels of one
+  int nfull, ngf;          // FP32: whole runs per summation block, groups of whole runs
+  int max_nf;              // FP32: most fields of a sub
+  int spw, njobs;          // FP64: 32-voxel steps per warp, jobs
+  const SumSub* subs;
+  const int* sub_fields;
+  const SumTile* tiles;
+  const SumJob* jobs;
+  const int* map;          // [n_ent] bin of each output (64 per tile, 4 per job), -1: none
+  int n_ent, ent0;         // outputs, first output of the level in the launch
+  double* partial;         // [splits][n_ent]
+  double scale;            // msum = scale * sum
+};
+struct SumArgs {
+  const void* fields;      // source fields [.][fstride] real T
+  double* msum;
+  const SumLevel* lv;      // device, most work first
+  int n_lv;
+  int items;               // of all levels
+  int n_ent;
+  int smem;                // FP32: shared-memory bytes of a block
+  int accumulate;          // msum += instead of msum = (later x-slabs of one sum)
+};
 
 // ---------------------------------------------------------------- error handling
 void set_error(const std::string& msg);
@@ -152,27 +195,14 @@ template <typename T>
 bsp_status launch_twiddles(void* tw, int ng, cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (bispec_contract.cu)
-struct ContractArgs {
-  const void* fields;     // [ns][nvox] real T
-  long long nvox;
-  int ns;
-  const Tile* tiles;
-  const int2* pairs;      // (a, b)
-  const int* tile_map;    // [ntiles][16]
-  int ntiles;
-  double* partial;        // [gridx][ntiles][16]
-  int gridx;
-  double* msum;           // [n_out]
-  int n_out;
-  double scale;           // msum = scale * (sum over the evaluation grid)
-  int accumulate;         // reduce: msum += instead of msum = (later x-slabs of one sum)
-};
 template <typename T>
-bsp_status launch_contract_simt(const ContractArgs& a, cudaStream_t s);
-bsp_status launch_reduce_partials(const ContractArgs& a, cudaStream_t s);
-template <typename T>
-bsp_status launch_decimate(const void* src, int S, const int* shells, int nsh, void* dst, int g, int t, int n_sm,
-                           cudaStream_t s);
+bsp_status launch_contract_simt(const SumArgs& a, cudaStream_t s);
+bsp_status launch_reduce_sums(const SumArgs& a, cudaStream_t s);
+int sum_stage_bytes(int nf);  // shared memory of an FP32 block that stages nf fields
+// Split fields of a coarser level from the evaluation grid's (tensor-core plans whose Z pass does
+// not write them).
+bsp_status launch_decimate(const uint16_t* src, int S, const int* shells, int nsh, uint16_t* dst, int g, int t,
+                           int n_sm, cudaStream_t s);
 
 struct FinalizeArgs {
   const double* msum;

@@ -53,18 +53,11 @@ struct ContractLevel {
   std::vector<int> shells;    // global shell of each local field index
   std::vector<int> bins;      // kept bins (global indices, ascending) summed on this level
   bool top = false;           // uses the plan's fields directly (all shells, global indices)
-  void* fields = nullptr;     // [shells][g^3] for lower levels (split planes [2][shells][g^3] for
-                              // tensor-core plans)
+  void* fields = nullptr;     // tensor-core plans: split planes [2][shells][g^3] of a lower level
   int* d_shells = nullptr;    // source field of each destination field of the level sampling
   CUtensorMap tmap{};         // tensor-core plans: the level's split fields (under a memory
                               // budget: those of a full x-slab)
   CUtensorMap tmap_last{};    // under a memory budget: the last (shorter) x-slab's split fields
-  // CUDA-core contraction
-  Tile* d_tiles = nullptr;
-  int2* d_pairs = nullptr;
-  int* d_map = nullptr;       // [ntiles][16] global bin index or -1
-  int ntiles = 0, gridx = 0;
-  double* partial = nullptr;
   // tensor-core contraction
   int np = 0, kt = 0, n_tg = 0, gridy = 0;  // padded shells, pair tiles per tile group, tile groups
   long long vpb = 0;
@@ -132,6 +125,7 @@ struct bsp_plan {
   int nwxi = 0, nwyi = 0;
   int rmax = 0;
   std::vector<ContractLevel> levels;
+  SumArgs sums{}, sums_last{};  // CUDA-core contraction of every level; of the last x-slab
   // each level's side and bins before split-BF16 plans merge levels (every pair on its smallest
   // exact grid): the algorithm's work, which bsp_plan_stage_work counts
   std::vector<std::pair<int, std::vector<int>>> exact_levels;
@@ -207,10 +201,15 @@ void make_items_g(const std::vector<ShellGeom>& geom, int grid, const PassLines&
                   std::vector<Item>& xi, std::vector<Item>& yi, std::vector<Item>& zi);
 void make_items(const bsp_plan* p, const PassLines& lines, std::vector<Item>& xi,
                 std::vector<Item>& yi, std::vector<Item>& zi);
-void make_tiles(const std::vector<int>& ta, const std::vector<int>& tb, const std::vector<int>& tc,
-                std::vector<int2>& pairs, std::vector<Tile>& tiles, std::vector<int>& map,
-                const std::vector<int>* ids = nullptr);
-int pick_gridx_n(int n_sm, int ntiles, long long nvox);
+// Device tables of a CUDA-core contraction level over bins (a, b, c) sorted by (a, b, c), ids[i] (or i)
+// the output of bin i; the caller gives *l the sampling and the scale. make_sum_args divides the
+// levels' voxels over a launch and allocates its partial sums. Allocations are also appended to
+// `owned` if given.
+bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::vector<int>& tb,
+                          const std::vector<int>& tc, const std::vector<int>* ids, bool f64, long long nvox,
+                          SumLevel* l, std::vector<void*>* owned, cudaStream_t s);
+bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel> lv, const std::vector<long long>& nvox, int spw, bool f64,
+                         SumArgs* out, std::vector<void*>* owned, cudaStream_t s);
 // Pair groups of the tensor-core contraction of one level: the slots (f0, f1, f2, flags) of n_tg
 // tile groups of kt tiles, and where[i] = (tg * kt + j) * kTcSlots + slot for pair i.
 struct TcGrouping {
