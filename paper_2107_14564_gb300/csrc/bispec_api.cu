@@ -402,37 +402,52 @@ bsp_status ball_setup(bsp_plan* p, cudaStream_t s) {
 bsp_status grad_setup(bsp_plan* p, cudaStream_t s) {
   if (p->grad_ready) return BSP_OK;
   const int ns = p->ns;
-  p->adj_np = ns <= 32 ? 32 : 64;
+  p->adj_np = adjoint_padded_shells(ns);
   const int np = p->adj_np;
   // every unordered pair (x >= y) that is the complement of a bin position
   std::vector<int> pid((size_t)ns * ns, -1);
-  std::vector<int2> pairs;
-  auto pair_index = [&](int x, int y) {
+  struct Pair { int2 ab; int q0, q1; std::vector<std::vector<int>> bins; };  // bins[n]: those with third n
+  std::vector<Pair> all;
+  auto add = [&](int x, int y, int n, int t) {
     if (x < y) std::swap(x, y);
     int& e = pid[(size_t)x * ns + y];
-    if (e < 0) { e = (int)pairs.size(); pairs.push_back(make_int2(x, y)); }
-    return e;
-  };
-  std::vector<std::vector<int>> lists;
-  auto add = [&](int pr, int n, int t) {
-    const size_t e = (size_t)pr * np + n;
-    if (lists.size() <= e) lists.resize(e + 1);
-    lists[e].push_back(t);
+    if (e < 0) {
+      e = (int)all.size();
+      all.push_back({make_int2(x, y), n / 4, n / 4 + 1, std::vector<std::vector<int>>(np)});
+    }
+    Pair& q = all[e];
+    q.q0 = std::min(q.q0, n / 4);
+    q.q1 = std::max(q.q1, n / 4 + 1);
+    q.bins[n].push_back(t);
   };
   for (size_t t = 0; t < p->trips.size(); ++t) {
     const bsp_triplet& b = p->trips[t];
-    add(pair_index(b.b, b.c), b.a, (int)t);
-    add(pair_index(b.a, b.c), b.b, (int)t);
-    add(pair_index(b.a, b.b), b.c, (int)t);
+    add(b.b, b.c, b.a, (int)t);
+    add(b.a, b.c, b.b, (int)t);
+    add(b.a, b.b, b.c, (int)t);
   }
-  p->adj_npairs = (int)pairs.size();
-  p->adj_entries = p->adj_npairs * np;
-  lists.resize(p->adj_entries);
-  std::vector<int> ptr(p->adj_entries + 1, 0), idx;
-  for (int e = 0; e < p->adj_entries; ++e) {
-    ptr[e + 1] = ptr[e] + (int)lists[e].size();
-    idx.insert(idx.end(), lists[e].begin(), lists[e].end());
+  // the lists of launch_adjoint_products, each made even by a pair without bins
+  std::vector<int2> pairs;
+  std::vector<int> ptr(1, 0), idx;
+  const Pair none{make_int2(0, 0), 0, 0, std::vector<std::vector<int>>(np)};
+  auto place = [&](const Pair& q) {
+    pairs.push_back(q.ab);
+    for (const std::vector<int>& b : q.bins) {
+      idx.insert(idx.end(), b.begin(), b.end());
+      ptr.push_back((int)idx.size());
+    }
+  };
+  for (int k = 0; k < kAdjRanges; ++k) {
+    p->adj_lists.p[k] = (int)pairs.size();
+    for (const Pair& q : all) {
+      int first = 0;  // the first range that holds it
+      while (q.q0 < adj_range(first, np / 4).q0 || q.q1 > adj_range(first, np / 4).q1) ++first;
+      if (first == k) place(q);
+    }
+    if (pairs.size() % 2) place(none);
   }
+  p->adj_lists.p[kAdjRanges] = (int)pairs.size();
+  p->adj_entries = (int)pairs.size() * np;
   const double vc = pow(p->box_len / p->ng, 3.0);
   const double norm = vc * vc * vc / (p->box_len * p->box_len * p->box_len);
   std::vector<double> cnorm(p->trips.size());
@@ -717,6 +732,7 @@ bsp_status bsp_grad(bsp_plan* p, const void* spec, const double* dl_db, float* d
   if (!p || !spec || !dl_db || !dl_ddelta) return fail(BSP_ERR_INVALID_ARG, "NULL argument");
   if (p->prec == BSP_FP64 || p->dim == 2 || p->order == 4)
     return fail(BSP_ERR_NOT_SUPPORTED, "bsp_grad needs a 3D bispectrum plan in FP32 or mixed precision");
+  if (p->ns > 64) return fail(BSP_ERR_NOT_SUPPORTED, "gradient: at most 64 shells");
   if (!warp_fft_supported(p->ngs) || !warp_fft_supported(p->ng))
     return fail(BSP_ERR_NOT_SUPPORTED, "bsp_grad needs grid sides 2^p or 3 * 2^p in [128, 1024]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -747,7 +763,7 @@ bsp_status bsp_grad(bsp_plan* p, const void* spec, const double* dl_db, float* d
     if ((st = plan_passes<float>(p, spec, p->fields, s, nullptr, false, part)) != BSP_OK) return st;
     const long long nvox = (long long)p->slab_len(k) * p->ngs * p->ngs;
     st = launch_adjoint_products(static_cast<const float*>(p->fields), nvox, p->ns, p->adj_np, p->d_adj_pairs,
-                                 p->adj_npairs, p->d_w, p->d_gfields, p->n_sm, s);
+                                 p->adj_lists, p->d_w, p->d_gfields, p->n_sm, s);
     if (st != BSP_OK) return st;
     // forward transforms of G_n, kept on each shell's modes: conj(.) K (ng/S)^3 into the ng spectrum
     a.slab_x0 = p->slab_nx ? p->slab_x0(k) : 0;

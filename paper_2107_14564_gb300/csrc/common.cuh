@@ -262,7 +262,17 @@ bsp_status launch_reduce_tc_all(const TcBin* bins, int n, double* msum, cudaStre
 // ---------------------------------------------------------------- gradient (bispec_grad.cu)
 bsp_status launch_build_w(const double* g, const double* cnorm, const int* ptr, const int* idx, int n_entries,
                           float* W, cudaStream_t s);
+// The pairs of the adjoint products are listed by the range of quads of n (of NQ) their bins reach.
+constexpr int kAdjRanges = 5;
+struct AdjRange { int q0, q1; };
+__host__ __device__ constexpr AdjRange adj_range(int k, int nq) {  // the narrower ranges first
+  return k == 0 ? AdjRange{0, nq / 2} : k == 1 ? AdjRange{nq / 2, nq} : k == 2 ? AdjRange{0, nq - nq / 4}
+       : k == 3 ? AdjRange{nq / 4, nq} : AdjRange{0, nq};
+}
+struct AdjLists { int p[kAdjRanges + 1]; };  // list k: pairs p[k] .. p[k + 1] - 1, an even number
+// W rows of np = adjoint_padded_shells(ns) floats, in the order of `pairs` (a, b).
+int adjoint_padded_shells(int ns);
 bsp_status launch_adjoint_products(const float* fields, long long nvox, int ns, int np, const int2* pairs,
-                                   int npairs, const float* W, float* G, int n_sm, cudaStream_t s);
+                                   const AdjLists& lists, const float* W, float* G, int n_sm, cudaStream_t s);
 
 }  // namespace bsp

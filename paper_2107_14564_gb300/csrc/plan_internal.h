@@ -133,7 +133,8 @@ struct bsp_plan {
   // gradient resources (built by the first bsp_grad call)
   bool grad_ready = false;
   bool ball_ready = false;
-  int adj_np = 0, adj_npairs = 0, adj_entries = 0;
+  int adj_np = 0, adj_entries = 0;
+  AdjLists adj_lists{};
   int2* d_adj_pairs = nullptr;
   int* d_w_ptr = nullptr;
   int* d_w_idx = nullptr;
