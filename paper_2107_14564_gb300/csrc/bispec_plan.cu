@@ -47,25 +47,22 @@ int fft_lines_for(int len, int prec) {
   return l < 1 ? 1 : l;
 }
 
-// Lines per block of the generic passes: as many as a block holds, fewer where a pass has too few lines
-// to give every SM a block that way, but at least 4 (2 in the Z pass, whose lines are contiguous) so
-// that accesses along k_z keep whole sectors. A 15-ring estimate at Ng = 384 (15 blocks of up to 31 x
-// 96 points a pass before) went from 51.5 to 37.6 us; two, four and eight blocks per SM gave
-// 43.7, 53.2 and 60.2 us, since a block of few lines takes as long as one of some more.
-static int spread(long long lines, int most, int least, int n_sm) {
-  return (int)std::min<long long>(most, std::max<long long>(least, (lines + n_sm - 1) / n_sm));
-}
-
+// Lines per block of the generic passes: as many as a block holds (a block never takes lines of two k_y or
+// x), fewer where a 2D pass has too few lines to give every SM a block that way, but at least 4 (2 along
+// the contiguous axis) so that accesses along k_y keep whole sectors. A 15-ring estimate at Ng = 384
+// (15 blocks of up to 31 x 96 points a pass before) went from 51.5 to 37.6 us; two, four and eight
+// blocks per SM gave 43.7, 53.2 and 60.2 us, since a block of few lines takes as long as one of some
+// more; for the same reason 3D passes, whose blocks are many, keep theirs whole.
 PassLines pass_lines(const bsp_plan* p, int prec) {
   const int most = fft_lines_for(p->ngs, prec), most_z = fft_lines_for(p->ngs / 2, prec);
-  long long x = 0, y = 0, z = 0;
-  for (const ShellGeom& g : p->geom) {
-    x += p->dim == 2 ? g.r : (long long)g.r * g.r * 3 / 2;  // lines (k_y, k_z >= 0) that meet the ball
-    y += (long long)p->ngs * g.r;
-    z += p->dim == 2 ? p->ngs : (long long)p->ngs * p->ngs;
-  }
-  const int n_sm = std::max(1, p->n_sm);
-  return {spread(x, most, 4, n_sm), spread(y, most, 4, n_sm), spread(z, most_z, 2, n_sm)};
+  if (p->dim == 3) return {most, most, most_z};
+  const long long n_sm = std::max(1, p->n_sm);
+  long long x = 0;
+  for (const ShellGeom& g : p->geom) x += g.r;
+  auto spread = [&](long long lines, int top, int least) {
+    return (int)std::min<long long>(top, std::max<long long>(least, (lines + n_sm - 1) / n_sm));
+  };
+  return {spread(x, most, 4), most, spread((long long)p->ns * p->ngs, most_z, 2)};
 }
 
 // Work items of the three passes for shells `geom` on a grid of side `grid`.
