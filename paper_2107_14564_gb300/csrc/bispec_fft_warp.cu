@@ -28,23 +28,6 @@ constexpr int kLines = 8;           // lines per X/Y block
 constexpr int kZThreads = 256;      // 8 warps, one line at a time each
 constexpr int kTileLd = kLines + 1; // padded tile row (complex)
 
-// Placement of point i in the per-line exchange buffers, chosen per length and radix list by
-// counting the shared-memory wavefronts of every stage's load and store pattern (64-bit accesses,
-// two half-warp phases): length 384 permutes i by i XOR ((i >> 3) & 15) (no extra space), 96 is
-// unpadded, the others get one spare slot every 2^shift points (shift 2 for 64, else 4).
-template <int N> struct Pad {
-  static constexpr bool kXor = N == 384;
-  static constexpr int shift = (kXor || N == 96) ? 0 : (N == 64 ? 2 : 4);
-};
-template <int N> __device__ __forceinline__ int padn(int i) {
-  if constexpr (Pad<N>::kXor) return i ^ ((i >> 3) & 15);
-  return Pad<N>::shift ? i + (i >> Pad<N>::shift) : i;
-}
-template <int N> __host__ __device__ constexpr int pad_len() { return Pad<N>::shift ? N + (N >> Pad<N>::shift) : N; }
-// Line stride of the X/Y buffers: 2 mod 16 complex, so the transposed read-out (8 lines x 2
-// consecutive points per half-warp) hits 16 distinct bank pairs.
-template <int N> __host__ __device__ constexpr int line_ld() { return pad_len<N>() + ((18 - pad_len<N>() % 16) % 16); }
-
 // Radix list and lanes per line of each supported length: every radix divides the points per
 // lane E = N / LPL, so each lane runs E / R whole butterflies per stage. Lengths 3 * 2^p use the
 // radix-6 and radix-12 butterflies: one exchange fewer than radix 3 followed by radices 2 to 4.
@@ -58,6 +41,56 @@ template <> struct Radices<384> { static constexpr int lpl = 16, n = 3; static c
 template <> struct Radices<512> { static constexpr int lpl = 32, n = 3; static constexpr int r[3] = {8, 8, 8}; };
 template <> struct Radices<768> { static constexpr int lpl = 32, n = 3; static constexpr int r[3] = {8, 8, 12}; };
 template <> struct Radices<1024> { static constexpr int lpl = 32, n = 4; static constexpr int r[4] = {8, 8, 8, 2}; };
+
+// Placement of point i in the exchange after stage S (sub-transforms of length ns, radix R): add spare
+// slots every `group` points, chosen per exchange by counting the shared-memory wavefronts of its
+// stores and loads (64-bit accesses, two half-warp phases) so that no access conflicts:
+//   * the first exchange stores runs R apart: one spare slot every 16 points spreads them;
+//   * with 1 < ns < 16 a half-warp stores 16 / ns runs of ns points, ns R apart: ns spare slots every
+//     ns R points put the runs side by side;
+//   * later exchanges move whole half-warps.
+// All of it folds into constants, the lane's own part aside. One padding for every exchange of a
+// length left 25% (192, 256) to 100% (96) more wavefronts, and these passes are bound by that pipe (Z
+// 97% busy): estimates at Ng = 256 and 24 shells 1.53 -> 1.48 ms (FP32), 0.957 -> 0.907 (split BF16, host
+// buffers), the shell fields at Ng = 384 and 8 shells 847 -> 818 us. XOR permutations without
+// conflicts cost more address arithmetic than they saved at 192 points (868 us).
+// The X/Y passes keep one placement from 384 points on, where longer lines would cost resident
+// blocks: 384 permutes i by i XOR ((i >> 3) & 15) (no extra space, no conflicts), the others spare one
+// slot every 16 points.
+template <int N>
+__host__ __device__ constexpr int sub_len(int S) {
+  int ns = 1;
+  for (int s = 0; s < S; ++s) ns *= Radices<N>::r[s];
+  return ns;
+}
+// Z: buffers of the Z passes (the half-warp holds two lines of 96 points, see z_line_ld).
+template <int N, int S, bool Z> struct Place {
+  static constexpr int ns = sub_len<N>(S);
+  static constexpr bool perm = !Z && N == 384;
+  static constexpr bool runs = S > 0 && ns < 16 && (Z || N <= 256);
+  static constexpr int group = N == 96 ? (S == 0 ? N : 24) : runs ? ns * Radices<N>::r[S] : 16;
+  static constexpr int add = N == 96 ? (S == 0 ? 0 : 14) : runs ? ns : 1;
+  static constexpr int len = perm ? N : N + add * ((N - 1) / group);
+  static __device__ __forceinline__ int at(int i) { return perm ? i ^ ((i >> 3) & 15) : i + add * (i / group); }
+};
+// Placement of the X/Y passes' output points.
+template <int N> __device__ __forceinline__ int padn(int i) { return N == 384 ? i ^ ((i >> 3) & 15) : i + (i >> 4); }
+template <int N, bool Z> __host__ __device__ constexpr int pad_len() {
+  int m = N == 384 && !Z ? N : N + (N >> 4);
+  m = Place<N, 0, Z>::len > m ? Place<N, 0, Z>::len : m;
+  return Place<N, 1, Z>::len > m ? Place<N, 1, Z>::len : m;
+}
+// Line stride of the X/Y buffers: 2 mod 16 complex, so the transposed read-out (8 lines x 2
+// consecutive points per half-warp) hits 16 distinct bank pairs.
+template <int N> __host__ __device__ constexpr int line_ld() {
+  return pad_len<N, false>() + ((18 - pad_len<N, false>() % 16) % 16);
+}
+// Line stride of the Z passes' buffers. With 8 lanes a line (96 points), a half-warp works on two
+// lines, 8 mod 16 complex apart: contiguous runs of 8 take turns. Its first exchange stores points 6
+// apart, all even or all odd; the odd lines swap even and odd places there (`par`).
+template <int N> __host__ __device__ constexpr int z_line_ld() {
+  return N == 96 ? pad_len<N, true>() + (24 - pad_len<N, true>() % 16) % 16 : pad_len<N, true>();
+}
 
 // Offset of stage S's twiddles in the stage-ordered table of length N: stage s (sub-transforms of
 // length NS_s = r_0 ... r_{s-1}, radix R_s) stores exp(2 pi i r k / (NS_s R_s)) at
@@ -109,8 +142,9 @@ __device__ __forceinline__ void stage_compute(float2* v, int lane, const float2*
   }
 }
 
-template <int N, int LPL, int R, int NS>
-__device__ __forceinline__ void stage_store(float2* buf, const float2* v, int lane) {
+template <int N, int LPL, int S, int NS, bool Z>
+__device__ __forceinline__ void stage_store(float2* buf, const float2* v, int lane, int par) {
+  constexpr int R = Radices<N>::r[S];
   constexpr int BPL = N / (R * LPL);
 #pragma unroll
   for (int b = 0; b < BPL; ++b) {
@@ -118,34 +152,53 @@ __device__ __forceinline__ void stage_store(float2* buf, const float2* v, int la
     const int k = j % NS;
     const int d = (j - k) * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) buf[padn<N>(d + r * NS)] = v[b * R + r];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (N == 96 && S == 0) {
+        buf[d + r + (r % 2 == 0 ? par : -par)] = v[b * R + r];  // d is even
+      } else if constexpr (Place<N, S, Z>::runs) {
+        // r NS stays below the group: the group index is that of the butterfly
+        buf[d + Place<N, S, Z>::add * (j / NS) + r * NS] = v[b * R + r];
+      } else {
+        buf[Place<N, S, Z>::at(d + r * NS)] = v[b * R + r];
+      }
+    }
   }
 }
 
-template <int N, int LPL, int R>
-__device__ __forceinline__ void stage_load(const float2* buf, float2* v, int lane) {
+template <int N, int LPL, int S, bool Z>
+__device__ __forceinline__ void stage_load(const float2* buf, float2* v, int lane, int par) {
+  constexpr int R = Radices<N>::r[S + 1];
   constexpr int BPL = N / (R * LPL);
+  if (N == 96 && S == 0) lane ^= par;
 #pragma unroll
   for (int b = 0; b < BPL; ++b) {
     const int j = lane + b * LPL;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[b * R + r] = buf[padn<N>(j + r * (N / R))];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (Place<N, S, Z>::perm) {
+        v[b * R + r] = buf[Place<N, S, Z>::at(j + r * (N / R))];
+      } else {
+        // lane + constant: lanes of one group of LPL points, or of 16 of them, share the spare slots
+        constexpr int G = Place<N, S, Z>::group, A = Place<N, S, Z>::add;
+        const int c = b * LPL + r * (N / R);
+        v[b * R + r] = buf[(G % LPL == 0 || G >= N ? lane : lane + A * (lane / G)) + c + A * (c / G)];
+      }
+    }
   }
 }
 
 // Inverse FFT of one line held by LPL lanes: on entry v[b R1 + r] = x[lane + b LPL + r N/R1],
 // on exit v[b RL + r] = y[lane + b LPL + r N/RL] (R1, RL the first and last radices).
-template <int N, int LPL, int S, int NS, bool POW = true>
-__device__ __forceinline__ void warp_fft_from(float2* v, float2* buf, int lane, const float2* stw) {
+template <int N, int LPL, int S, int NS, bool POW, bool Z>
+__device__ __forceinline__ void warp_fft_from(float2* v, float2* buf, int lane, const float2* stw, int par = 0) {
   constexpr int R = Radices<N>::r[S];
   stage_compute<N, LPL, R, NS, stage_off<N>(S), POW>(v, lane, stw);
   if constexpr (S + 1 < Radices<N>::n) {
-    constexpr int R2 = Radices<N>::r[S + 1];
     __syncwarp();
-    stage_store<N, LPL, R, NS>(buf, v, lane);
+    stage_store<N, LPL, S, NS, Z>(buf, v, lane, par);
     __syncwarp();
-    stage_load<N, LPL, R2>(buf, v, lane);
-    warp_fft_from<N, LPL, S + 1, NS * R, POW>(v, buf, lane, stw);
+    stage_load<N, LPL, S, Z>(buf, v, lane, par);
+    warp_fft_from<N, LPL, S + 1, NS * R, POW, Z>(v, buf, lane, stw, par);
   }
 }
 
@@ -278,7 +331,7 @@ __global__ void __launch_bounds__(XY<N>::kThreads, xy_min_blocks<N>()) xy_warp_k
         }
       __syncthreads();  // every line has read the tile its buffers overlay
       float2* buf = bufs + (size_t)l * kBufLd;
-      warp_fft_from<N, LPL, 0, 1>(v, buf, lane, tw);
+      warp_fft_from<N, LPL, 0, 1, true, false>(v, buf, lane, tw);
       constexpr int RL = last_radix<N>();
       constexpr int BPLL = N / (RL * LPL);
       __syncwarp();
@@ -320,7 +373,7 @@ __global__ void __launch_bounds__(kZThreads, z_min_blocks<S>()) z_warp_kernel(Pa
   constexpr int LPL = Radices<M>::lpl;
   constexpr int LPW = 32 / LPL;  // lines per warp at a time
   constexpr int E = M / LPL;
-  constexpr int kBufLd = pad_len<M>();
+  constexpr int kBufLd = z_line_ld<M>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* tw = reinterpret_cast<float2*>(smem_raw);  // M entries: stage twiddles of length M
   float2* wk = tw + M;                               // M entries: exp(2 pi i k / S), k < M
@@ -365,7 +418,7 @@ __global__ void __launch_bounds__(kZThreads, z_min_blocks<S>()) z_warp_kernel(Pa
         const float2 o = c_mul(make_float2(xk.x - xm.x, xk.y + xm.y), wk[k]);  // (X[k] - conj X[M-k]) W^k
         v[b * R1 + rr] = make_float2(e.x - o.y, e.y + o.x);                    // e + i o
       }
-    warp_fft_from<M, LPL, 0, 1, false>(v, buf, lane, tw);
+    warp_fft_from<M, LPL, 0, 1, false, true>(v, buf, lane, tw, sub & 1);
     const long long off = (long long)n * S * per + xyl * S;  // first voxel of the line
     if (a.split_lo == 0) {
       float2* dst = reinterpret_cast<float2*>(static_cast<float*>(a.fields) + off);
@@ -464,7 +517,7 @@ __global__ void __launch_bounds__(kZThreads) zf_warp_kernel(PassArgs a, const fl
   constexpr int LPL = Radices<S>::lpl;
   constexpr int LPW = 32 / LPL;
   constexpr int E = S / LPL;
-  constexpr int kBufLd = pad_len<S>();
+  constexpr int kBufLd = z_line_ld<S>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* tw = reinterpret_cast<float2*>(smem_raw);  // stage twiddles of length S
   float2* bufs = tw + S;
@@ -495,7 +548,7 @@ __global__ void __launch_bounds__(kZThreads) zf_warp_kernel(PassArgs a, const fl
     for (int b = 0; b < BPL; ++b)
 #pragma unroll
       for (int rr = 0; rr < R1; ++rr) v[b * R1 + rr] = make_float2(src[lane + b * LPL + rr * (S / R1)], 0.f);
-    warp_fft_from<S, LPL, 0, 1>(v, buf, lane, tw);
+    warp_fft_from<S, LPL, 0, 1, true, true>(v, buf, lane, tw);
     float2* dst = static_cast<float2*>(a.g2) + g.g2_off + xy * r;
 #pragma unroll
     for (int b = 0; b < BPLL; ++b)
@@ -552,7 +605,7 @@ __global__ void __launch_bounds__(XY<N>::kThreads) xyf_warp_kernel(PassArgs a, f
 #pragma unroll
       for (int rr = 0; rr < R1; ++rr) v[b * R1 + rr] = tile[(lane + b * LPL + rr * (N / R1)) * kTileLd + l];
     float2* buf = bufs + (size_t)l * kBufLd;
-    warp_fft_from<N, LPL, 0, 1>(v, buf, lane, tw);
+    warp_fft_from<N, LPL, 0, 1, true, false>(v, buf, lane, tw);
     constexpr int RL = last_radix<N>();
     constexpr int BPLL = N / (RL * LPL);
     __syncwarp();
@@ -607,7 +660,7 @@ bsp_status launch_xyf(const PassArgs& a, int n_items, float scale, cudaStream_t 
 template <int S>
 bsp_status launch_zf(const PassArgs& a, const float* gfield, long long n_lines, int n_sm, cudaStream_t s) {
   constexpr int LPW = 32 / Radices<S>::lpl;
-  const size_t smem = ((size_t)S + (size_t)(kZThreads / 32) * LPW * pad_len<S>()) * sizeof(float2);
+  const size_t smem = ((size_t)S + (size_t)(kZThreads / 32) * LPW * z_line_ld<S>()) * sizeof(float2);
   BSP_CUDA(cudaFuncSetAttribute(zf_warp_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, zf_warp_kernel<S>, kZThreads, smem));
@@ -640,7 +693,7 @@ template <int S>
 bsp_status launch_z(const PassArgs& a, long long n_lines, int n_sm, cudaStream_t s) {
   constexpr int M = S / 2;
   constexpr int LPW = 32 / Radices<M>::lpl;
-  const size_t smem = ((size_t)2 * M + (size_t)(kZThreads / 32) * LPW * pad_len<M>()) * sizeof(float2) +
+  const size_t smem = ((size_t)2 * M + (size_t)(kZThreads / 32) * LPW * z_line_ld<M>()) * sizeof(float2) +
                       (a.n_zlev > 0 ? (size_t)S * sizeof(uint32_t) : 0);
   auto kern = a.slab_nx > 0 ? z_warp_kernel<S, true> : z_warp_kernel<S, false>;
   BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
