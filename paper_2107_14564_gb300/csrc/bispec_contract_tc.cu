@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
       ptx::mbar_init(&full[i], 1);
       ptx::mbar_init(&mmad[i], KT);
     }
-    for (int i = 0; i < L::kNA; ++i) ptx::mbar_init(&gen[i], kTcGenWarps);
+    for (int i = 0; i < L::kNA; ++i) ptx::mbar_init(&gen[i], kTcGenWarps / 2);
     ptx::mbar_init(flushed, kTcGenWarps);
     ptx::mbar_init(drain, KT);
     *abort_flag = 0;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
     // ------------------------------------------------------------ generators
     const int quarter = warp & 3;      // TMEM lanes 32 quarter .. + 31
     const int half = (warp >> 2) & 1;  // lanes 32 quarter + 16 half .. + 15
-    const int kg = warp >> 3;          // K steps 2 kg, 2 kg + 1 of every chunk
+    const int cg = warp >> 3;          // chunks of this parity; accumulators of tiles cg, cg + 2
     const int r = lane >> 2;           // slot row: Ph in lane r, Pl in lane r + 8 of the half
     const int t4 = lane & 3;           // voxels 4 t4 .. 4 t4 + 3 of a K step
     const int slot = quarter * 16 + half * 8 + r;
@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
     const bool warp_active = __any_sync(0xffffffffu, active);
     const uint32_t lane_base = (uint32_t)(32 * quarter + 16 * half) << 16;
     // byte offsets, within a B stage's high plane, of this thread's 8 bytes of field f in K step
-    // 2 kg + k: row f of the 128-byte-swizzled box, 16-byte column (2 (2 kg + k) + t4 / 2) XOR (f & 7)
+    // k < 2: row f of the 128-byte-swizzled box, 16-byte column (2 k + t4 / 2) XOR (f & 7); K step k + 2
+    // lies 4 columns on, at the offset XOR 64
     int off[L::kFields][2];
     {
       const int fs[3] = {grp.x, grp.y, grp.z};
@@ -252,11 +253,11 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           const int n = fs[f];
-          const int col = (2 * (2 * kg + k) + (t4 >> 1)) ^ (n & 7);
+          const int col = (2 * k + (t4 >> 1)) ^ (n & 7);
           off[f][k] = (n >> 3) * 1024 + (n & 7) * 128 + (col << 4) + ((t4 & 1) << 3);
         }
     }
-    // tiles whose accumulators this warp reads back: j = kg, kg + 2; their run sums are kept as
+    // tiles whose accumulators this warp reads back: j = cg, cg + 2; their run sums are kept as
     // compensated FP32 pairs in this block's rows of the partial-sum buffer (L2-resident, one
     // owner per entry), read, added to and written back once per run
     constexpr int kMine = (KT + 1) / 2;
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
     auto flush = [&]() {
 #pragma unroll
       for (int m = 0; m < kMine; ++m) {
-        const int j = kg + 2 * m;
+        const int j = cg + 2 * m;
         if (j >= KT) break;
         float v[kAccN];
 #pragma unroll
@@ -300,99 +301,94 @@ __global__ void __launch_bounds__(tc_threads<KT>(), 1)
       }
       have = true;
     };
-    // Hand a finished A stage to the MMA warp once its tensor-memory stores have landed. Done one
-    // chunk late, so the store latency overlaps the next chunk's arithmetic. One arrival per warp.
-    auto publish = [&](int s) {
-      ptx::tmem_st_wait();
+    // Read the accumulators back once every MMA of the chunks before `next` is done.
+    auto close_run = [&](int next) {
+      const int j = next - 1;
+      if (!tc_wait(&mmad[j % L::kNB], (uint32_t)((j / L::kNB) & 1), abort_flag)) return false;
+      ptx::tc_fence_after();
+      if (warp_active) flush();
+      return true;
+    };
+    // ... between two runs, then let the MMA warps restart the accumulators.
+    int runs = 0;  // read back so far
+    auto end_run = [&]() {
+      if (!close_run(++runs * kTcRun)) return false;
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&gen[s]);
+      if (lane == 0) ptx::mbar_arrive(flushed);
+      return true;
     };
-    int sa = 0, sa_prev = L::kNA - 1;  // i % kNA and (i - 1) % kNA, kept as counters
-    for (int i = 0; i < nchunks; ++i) {
+    int sa = cg % L::kNA;  // i % kNA, kept as a counter
+    for (int i = cg; i < nchunks; i += 2) {
       const int sb = i % L::kNB;
-      if (!tc_wait(&full[sb], (uint32_t)((i / L::kNB) & 1), abort_flag)) {
+      if ((i >= (runs + 1) * kTcRun && !end_run()) || !tc_wait(&full[sb], (uint32_t)((i / L::kNB) & 1), abort_flag)) {
         *abort_flag = 1;
         failed = true;
         break;
       }
       const unsigned char* st = bs + (size_t)sb * L::kBStage;
-      // this slot's fields for 4 voxels of each of 2 K steps (high and low planes)
-      uint2 fh[2][L::kFields], fl[2][L::kFields];
-      if (warp_active) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
+      for (int h = 0; h < 2; ++h) {  // K steps 2 h, 2 h + 1
+        // this slot's fields for 4 voxels of each of 2 K steps (high and low planes)
+        uint2 fh[2][L::kFields], fl[2][L::kFields];
+        // A operand: the slot's KT pair products; tile 0 (f0, s ? f1 : f0), 1 (f0, f2), 2 (f1, f2)
+        uint32_t pv[KT][8];
+        if (warp_active) {
 #pragma unroll
-          for (int f = 0; f < L::kFields; ++f) {
-            fh[k][f] = *reinterpret_cast<const uint2*>(st + off[f][k]);
-            fl[k][f] = *reinterpret_cast<const uint2*>(st + L::kBPlane + off[f][k]);
-          }
-      }
-      // the previous chunk's A stores have landed while the loads were in flight: hand it over
-      if (i > 0) publish(sa_prev);
-      // A operand: the slot's KT pair products; tile 0 (f0, s ? f1 : f0), 1 (f0, f2), 2 (f1, f2)
-      uint32_t pv[KT][8];
-      if (warp_active) {
+          for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
+            for (int f = 0; f < L::kFields; ++f) {
+              fh[k][f] = *reinterpret_cast<const uint2*>(st + (off[f][k] ^ (64 * h)));
+              fl[k][f] = *reinterpret_cast<const uint2*>(st + L::kBPlane + (off[f][k] ^ (64 * h)));
+            }
 #pragma unroll
-          for (int j = 0; j < KT; ++j) {
-            const int ia = j == 2 ? 1 : 0;
-            const int ib = j == 0 ? 1 : 2;
-            uint2 bh = fh[k][ib < L::kFields ? ib : 0], bl = fl[k][ib < L::kFields ? ib : 0];
-            if (j == 0 && !sel1) { bh = fh[k][0]; bl = fl[k][0]; }
-            ptx::bf16x2_pair_product(fh[k][ia].x, fl[k][ia].x, bh.x, bl.x, pv[j][4 * k + 0], pv[j][4 * k + 2]);
-            ptx::bf16x2_pair_product(fh[k][ia].y, fl[k][ia].y, bh.y, bl.y, pv[j][4 * k + 1], pv[j][4 * k + 3]);
-          }
-      }
-      if (i > 0 && i % kTcRun == 0) {
-        // chunk i - 1 closed a run: wait for its MMAs (and with them every earlier one), read
-        // the accumulators back, then let the MMA warps restart them
-        const int j = i - 1;
-        if (!tc_wait(&mmad[j % L::kNB], (uint32_t)((j / L::kNB) & 1), abort_flag)) {
-          *abort_flag = 1;
-          failed = true;
-          break;
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int j = 0; j < KT; ++j) {
+              const int ia = j == 2 ? 1 : 0;
+              const int ib = j == 0 ? 1 : 2;
+              uint2 bh = fh[k][ib < L::kFields ? ib : 0], bl = fl[k][ib < L::kFields ? ib : 0];
+              if (j == 0 && !sel1) { bh = fh[k][0]; bl = fl[k][0]; }
+              ptx::bf16x2_pair_product(fh[k][ia].x, fl[k][ia].x, bh.x, bl.x, pv[j][4 * k + 0], pv[j][4 * k + 2]);
+              ptx::bf16x2_pair_product(fh[k][ia].y, fl[k][ia].y, bh.y, bl.y, pv[j][4 * k + 1], pv[j][4 * k + 3]);
+            }
         }
-        ptx::tc_fence_after();
-        if (warp_active) flush();
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(flushed);
-      }
-      if (i >= L::kNA) {
-        const int j = i - L::kNA;  // the chunk that last used A stage sa
-        if (!tc_wait(&mmad[j % L::kNB], (uint32_t)((j / L::kNB) & 1), abort_flag)) {
-          *abort_flag = 1;
-          failed = true;
-          break;
+        if (h == 0) {
+          if (i >= L::kNA) {
+            const int j = i - L::kNA;  // the chunk that last used A stage sa
+            if (!tc_wait(&mmad[j % L::kNB], (uint32_t)((j / L::kNB) & 1), abort_flag)) {
+              *abort_flag = 1;
+              failed = true;
+              break;
+            }
+          }
+          ptx::tc_fence_after();
+        }
+        if (warp_active) {
+#pragma unroll
+          for (int j = 0; j < KT; ++j)
+            ptx::tmem_st_16x256b_x2(tmem + lane_base + (uint32_t)(L::kAStage * sa + 32 * j + 16 * h), pv[j]);
         }
       }
-      ptx::tc_fence_after();
-      if (warp_active) {
-#pragma unroll
-        for (int j = 0; j < KT; ++j)
-          ptx::tmem_st_16x256b_x2(tmem + lane_base + (uint32_t)(L::kAStage * sa + 32 * j + 16 * kg), pv[j]);
-      }
-      sa_prev = sa;
-      if (++sa == L::kNA) sa = 0;
+      if (failed) break;
+      // hand the A stage to the MMA warps once its tensor-memory stores have landed; one arrival per warp
+      ptx::tmem_st_wait();
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&gen[sa]);
+      sa += 2;
+      if (sa >= L::kNA) sa -= L::kNA;
     }
-    if (!failed && nchunks > 0) publish((nchunks - 1) % L::kNA);
-    if (!failed && nchunks > 0) {
-      const int last = nchunks - 1;
-      if (tc_wait(&mmad[last % L::kNB], (uint32_t)((last / L::kNB) & 1), abort_flag)) {
-        ptx::tc_fence_after();
-        if (warp_active) flush();
-      } else {
-        failed = true;
-      }
-    }
+    // a last run of one chunk is not this warp's to make, but ends the run before it
+    if (!failed && nchunks > 0 && (nchunks - 1) / kTcRun > runs) failed = !end_run();
+    if (!failed && nchunks > 0) failed = !close_run(nchunks);
+    if (failed) *abort_flag = 1;
     if (failed) ptx::tmem_st_wait();
     if (nchunks == 0 && active) {
       // a block without voxels (a short x-slab of a budgeted plan) still owns its partial sums
 #pragma unroll
       for (int m = 0; m < kMine; ++m) {
-        const int j = kg + 2 * m;
+        const int j = cg + 2 * m;
         if (j >= KT) break;
         float2* out = a.partial + ((((size_t)blockIdx.y * a.n_tg + tg) * KT + j) * kTcSlots + slot) * NP;
 #pragma unroll
