@@ -381,7 +381,7 @@ bsp_status ball_setup(bsp_plan* p, cudaStream_t s) {
   ball[0].qlo = (int)p->q[0];
   ball[0].qhi = (int)p->q[p->ns];
   ball[0].r = (int)isqrt_ll(p->q[p->ns] - 1) + 1;
-  ball[0].pad = 0;
+  ball[0].rp = row_pitch(ball[0].r);
   ball[0].g1_off = 0;
   ball[0].g2_off = 0;
   std::vector<Item> bx, by, bz;
@@ -391,9 +391,9 @@ bsp_status ball_setup(bsp_plan* p, cudaStream_t s) {
   if ((st = dev_upload(p, ball, &p->d_ball, s)) != BSP_OK) return st;
   if ((st = dev_upload(p, bx, &p->d_bxi, s)) != BSP_OK) return st;
   if ((st = dev_upload(p, by, &p->d_byi, s)) != BSP_OK) return st;
-  const long long r = ball[0].r;
-  if ((st = dev_alloc(p, (size_t)p->ng * (2 * r - 1) * r * sizeof(float2), &p->g1b)) != BSP_OK) return st;
-  if ((st = dev_alloc(p, (size_t)p->ng * p->ng * r * sizeof(float2), &p->g2b)) != BSP_OK) return st;
+  const long long r = ball[0].r, rp = ball[0].rp;
+  if ((st = dev_alloc(p, (size_t)p->ng * (2 * r - 1) * rp * sizeof(float2), &p->g1b)) != BSP_OK) return st;
+  if ((st = dev_alloc(p, (size_t)p->ng * p->ng * rp * sizeof(float2), &p->g2b)) != BSP_OK) return st;
   p->ball_ready = true;
   return BSP_OK;
 }

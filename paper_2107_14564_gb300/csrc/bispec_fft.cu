@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kFftThreads) xpass_kernel(PassArgs a, int max_
   for (int idx = threadIdx.x; idx < S * nl; idx += blockDim.x) {
     const int kzl = idx % nl;
     const int x = idx / nl;
-    g1[((long long)x * w + jy) * r + it.v0 + kzl] = buf[kzl * S + x];
+    g1[((long long)x * w + jy) * g.rp + it.v0 + kzl] = buf[kzl * S + x];
   }
 }
 
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kFftThreads) ypass_kernel(PassArgs a, int max_
     const int kz = it.v0 + kzl;
     if (ky * ky + kz * kz < g.qhi) {
       const int iy = ky < 0 ? ky + ng : ky;
-      buf[kzl * ng + iy] = g1[((long long)x * w + jy) * r + kz];
+      buf[kzl * ng + iy] = g1[((long long)x * w + jy) * g.rp + kz];
     }
   }
   __syncthreads();
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kFftThreads) ypass_kernel(PassArgs a, int max_
   for (int idx = threadIdx.x; idx < ng * nl; idx += blockDim.x) {
     const int kzl = idx % nl;
     const int y = idx / nl;
-    g2[((long long)x * ng + y) * r + it.v0 + kzl] = buf[kzl * ng + y];
+    g2[((long long)x * ng + y) * g.rp + it.v0 + kzl] = buf[kzl * ng + y];
   }
 }
 
@@ -204,11 +204,11 @@ __global__ void __launch_bounds__(kFftThreads) zpass_kernel(PassArgs a, int max_
   __syncthreads();
   const int r = g.r;
   const int x = it.u;
-  const C* g2 = static_cast<const C*>(a.g2) + g.g2_off + ((long long)x * ng + it.v0) * r;
+  const C* g2 = static_cast<const C*>(a.g2) + g.g2_off + ((long long)x * ng + it.v0) * g.rp;
   for (int idx = threadIdx.x; idx < r * nl; idx += blockDim.x) {
     const int l = idx / r;
     const int k = idx - l * r;
-    buf[l * M + k] = g2[idx];
+    buf[l * M + k] = g2[l * g.rp + k];
   }
   __syncthreads();
   const int half = M / 2 + 1;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kFftThreads) zpass_kernel(PassArgs a, int max_
 // Item (n, -, v0, cnt): the k_y lines v0 .. v0 + cnt - 1 of ring n (|k_y| < r, k_y >= 0 on the
 // halved axis). Gathers the ring's modes along k_x (|k_x| < r) from the 2D half spectrum
 // [ng][ng/2 + 1], transforms along x on the evaluation grid (length ngs) and writes
-// G[g1_off + x r + k_y], the rows the C2R along y then reads.
+// G[g1_off + x rp + k_y], the rows the C2R along y then reads.
 template <typename T>
 __global__ void __launch_bounds__(kFftThreads) ring_xpass_kernel(PassArgs a, int max_lines) {
   using C = cplx<T>;
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kFftThreads) ring_xpass_kernel(PassArgs a, int
   for (int idx = threadIdx.x; idx < S * nl; idx += blockDim.x) {
     const int l = idx % nl;
     const int x = idx / nl;
-    out[(long long)x * r + it.v0 + l] = buf[l * S + x];
+    out[(long long)x * g.rp + it.v0 + l] = buf[l * S + x];
   }
 }
 

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(XY<N>::kThreads, xy_min_blocks<N>()) xy_warp_k
         const int ky = row - (r - 1);
         const int kz = it.v0 + l;
         const bool in = l < it.cnt && ky * ky + kz * kz < g.qhi;
-        const float2* src = in ? g1 + ((long long)x * w + row) * r + kz : g1;
+        const float2* src = in ? g1 + ((long long)x * w + row) * g.rp + kz : g1;
         ptx::cp_async8_zfill(tile + row * kTileLd + l, src, in ? 8u : 0u);
       }
     }
@@ -345,16 +345,153 @@ __global__ void __launch_bounds__(XY<N>::kThreads, xy_min_blocks<N>()) xy_warp_k
     float2* out;
     long long row_stride;
     if (XPASS) {
-      out = static_cast<float2*>(a.g1) + g.g1_off + (long long)(it.u + r - 1) * r + it.v0;
-      row_stride = (long long)w * r;
+      out = static_cast<float2*>(a.g1) + g.g1_off + (long long)(it.u + r - 1) * g.rp + it.v0;
+      row_stride = (long long)w * g.rp;
     } else {
-      out = static_cast<float2*>(a.g2) + g.g2_off + (long long)it.u * N * r + it.v0;
-      row_stride = r;
+      out = static_cast<float2*>(a.g2) + g.g2_off + (long long)it.u * N * g.rp + it.v0;
+      row_stride = g.rp;
     }
     for (int idx = tid; idx < N * kLines; idx += NT) {
       const int l = idx & (kLines - 1);
       const int y = idx >> 3;
       if (l < it.cnt) out[y * row_stride + l] = bufs[(size_t)l * kBufLd + padn<N>(y)];
+    }
+  }
+}
+
+// ---------------------------------------------------------------- X and Y passes, lines in registers
+// A warp takes 4 neighbouring k_z lines of an item, 8 lanes a line: thread (line l = t & 3, lane t >> 2)
+// loads and stores its E = N / 8 points straight from and to global memory, 32 bytes of k_z at a time,
+// so only the exchanges between stages use shared memory and no block barrier is needed. The kernel
+// above passes every point through a staged tile and the line buffers on top (8 accesses a point
+// instead of 4, and their index arithmetic).
+// Exchange placement: the first exchange stores points R apart, one spare slot every R points makes
+// them R + 1 apart; later ones move runs of at least 4. With lines 4 mod 16 complex apart, the 4 lines x
+// 4 lanes of a half-warp then meet 16 different banks.
+// Taken where it is the faster one (xy_in_lines), us per pass, this kernel / the one above: Y 128 points
+// 28 / 43 (30 shells), 192: 94 / 109 (24 shells), 256: 135 / 174 (16 shells), 384: 1147 / 1222 (32 shells), 512:
+// 1118 / 952 (10 shells); X 11.6 / 14.6, 36.5 / 42.6, 59.6 / 66.0, 641 / 464, 403 / 311. It bears whole sectors only:
+// with rows of k_z not padded to 64 bytes the Y pass of 384 points took 2285.
+constexpr bool xy_in_lines(int n, bool xpass) { return n <= (xpass ? 256 : 384); }
+template <int N> struct XYL {
+  static constexpr int kLpl = 8;
+  static constexpr int kE = N / kLpl;
+  static constexpr int kR0 = Radices<N>::r[0];
+  static constexpr int kLen = N + N / kR0;
+  static constexpr int kLd = kLen + (20 - kLen % 16) % 16;
+  static constexpr int kThreads = 128;
+  static constexpr int kBlocks = N <= 128 ? 6 : N <= 192 ? 5 : N <= 256 ? 4 : 3;  // as the points' registers allow
+  static constexpr size_t kSmem = ((size_t)N + (size_t)(kThreads / 32) * 4 * kLd) * sizeof(float2);
+};
+
+template <int N, int S, int NS>
+__device__ __forceinline__ void line_fft_from(float2* v, float2* buf, int lane, const float2* stw) {
+  constexpr int LPL = XYL<N>::kLpl;
+  constexpr int R = Radices<N>::r[S];
+  stage_compute<N, LPL, R, NS, stage_off<N>(S), true>(v, lane, stw);
+  if constexpr (S + 1 < Radices<N>::n) {
+    constexpr int R0 = XYL<N>::kR0;
+    constexpr int BPL = N / (R * LPL);
+    __syncwarp();
+#pragma unroll
+    for (int b = 0; b < BPL; ++b) {
+      const int j = lane + b * LPL;
+      const int k = j % NS;
+      const int d = (j - k) * R + k;
+#pragma unroll
+      for (int r = 0; r < R; ++r) buf[S == 0 ? (R0 + 1) * j + r : d + r * NS] = v[b * R + r];
+    }
+    __syncwarp();
+    constexpr int R2 = Radices<N>::r[S + 1];
+    constexpr int BPL2 = N / (R2 * LPL);
+#pragma unroll
+    for (int b = 0; b < BPL2; ++b)
+#pragma unroll
+      for (int r = 0; r < R2; ++r) {
+        const int c = b * LPL + r * (N / R2);  // a multiple of 8
+        v[b * R2 + r] = buf[S == 0 ? lane + lane / R0 + c + c / R0 : lane + c];
+      }
+    line_fft_from<N, S + 1, NS * R>(v, buf, lane, stw);
+  }
+}
+
+template <int N, bool XPASS>
+__global__ void __launch_bounds__(XYL<N>::kThreads, XYL<N>::kBlocks) xy_line_kernel(PassArgs a, int n_items) {
+  constexpr int LPL = XYL<N>::kLpl;
+  constexpr int E = XYL<N>::kE;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* tw = reinterpret_cast<float2*>(smem_raw);  // N entries
+  const int tid = threadIdx.x;
+  for (int i = tid; i < N; i += XYL<N>::kThreads) tw[i] = static_cast<const float2*>(a.stw)[i];
+  __syncthreads();
+  const int l = tid & 3;
+  const int lane = (tid & 31) >> 2;
+  float2* buf = tw + N + ((tid >> 5) * 4 + l) * XYL<N>::kLd;
+  constexpr int R1 = first_radix<N>(), BPL = N / (R1 * LPL);
+  constexpr int RL = last_radix<N>(), BPLL = N / (RL * LPL);
+  const int warps = (int)gridDim.x * (XYL<N>::kThreads / 32);
+  for (int u = blockIdx.x * (XYL<N>::kThreads / 32) + (tid >> 5); u < 2 * n_items; u += warps) {
+    const Item it = a.items[u >> 1];  // 8 lines: two units of 4
+    const int l0 = (u & 1) * 4;
+    if (l0 >= it.cnt) continue;
+    const ShellGeom g = a.geom[it.n];
+    const int r = g.r;
+    const int w = 2 * r - 1;
+    const int kz = it.v0 + l0 + l;
+    const bool on = l0 + l < it.cnt;
+    float2 v[E];
+    if (XPASS) {
+      const float2* spec = static_cast<const float2*>(a.spec);
+      const int ng = a.ng;  // side of the input spectrum's grid
+      const int ky = it.u;
+      const int hz = ng / 2 + 1;
+      const int q0 = ky * ky + kz * kz;
+      const float2* line = spec + (long long)(ky < 0 ? ky + ng : ky) * hz + kz;
+#pragma unroll
+      for (int b = 0; b < BPL; ++b)
+#pragma unroll
+        for (int rr = 0; rr < R1; ++rr) {
+          const int pos = lane + b * LPL + rr * (N / R1);
+          const int mx = pos < N / 2 ? pos : pos - N;
+          const int q = q0 + mx * mx;
+          const bool in = on && q >= g.qlo && q < g.qhi;
+          float2 t = make_float2(0.f, 0.f);
+          if (in) t = spec ? line[(long long)(mx < 0 ? mx + ng : mx) * ng * hz] : make_float2(1.f, 0.f);
+          if (a.rsd && in) {  // Kaiser factor (Eq. (3.4)) of the shell's modes, in FP32
+            const float fac = 1.0f + (float)a.beta * ((float)(kz * kz) / (float)q);
+            t.x *= fac;
+            t.y *= fac;
+          }
+          v[b * R1 + rr] = t;
+        }
+    } else {
+      const float2* line = static_cast<const float2*>(a.g1) + g.g1_off + ((long long)it.u * w + r - 1) * g.rp + kz;
+#pragma unroll
+      for (int b = 0; b < BPL; ++b)
+#pragma unroll
+        for (int rr = 0; rr < R1; ++rr) {
+          const int pos = lane + b * LPL + rr * (N / R1);
+          const int ky = pos < N / 2 ? pos : pos - N;
+          float2 t = make_float2(0.f, 0.f);
+          if (on && ky * ky + kz * kz < g.qhi) t = line[ky * g.rp];
+          v[b * R1 + rr] = t;
+        }
+    }
+    line_fft_from<N, 0, 1>(v, buf, lane, tw);
+    if (on) {
+      float2* out;
+      int stride;  // between points of the line
+      if (XPASS) {
+        out = static_cast<float2*>(a.g1) + g.g1_off + (long long)(it.u + r - 1) * g.rp + kz;
+        stride = w * g.rp;
+      } else {
+        out = static_cast<float2*>(a.g2) + g.g2_off + (long long)it.u * N * g.rp + kz;
+        stride = g.rp;
+      }
+#pragma unroll
+      for (int b = 0; b < BPLL; ++b)
+#pragma unroll
+        for (int rr = 0; rr < RL; ++rr) out[(long long)(lane + b * LPL + rr * (N / RL)) * stride] = v[b * RL + rr];
     }
   }
 }
@@ -405,7 +542,7 @@ __global__ void __launch_bounds__(kZThreads, z_min_blocks<S>()) z_warp_kernel(Pa
     const long long xy = SLAB ? (long long)a.slab_x0 * S + xyl : xyl;  // (x, y) on the grid
     const ShellGeom g = a.geom[n];
     const int r = g.r;
-    const float2* src = static_cast<const float2*>(a.g2) + g.g2_off + xy * r;
+    const float2* src = static_cast<const float2*>(a.g2) + g.g2_off + xy * g.rp;
     float2 v[E];
 #pragma unroll
     for (int b = 0; b < BPL; ++b)
@@ -549,7 +686,7 @@ __global__ void __launch_bounds__(kZThreads) zf_warp_kernel(PassArgs a, const fl
 #pragma unroll
       for (int rr = 0; rr < R1; ++rr) v[b * R1 + rr] = make_float2(src[lane + b * LPL + rr * (S / R1)], 0.f);
     warp_fft_from<S, LPL, 0, 1, true, true>(v, buf, lane, tw);
-    float2* dst = static_cast<float2*>(a.g2) + g.g2_off + xy * r;
+    float2* dst = static_cast<float2*>(a.g2) + g.g2_off + xy * g.rp;
 #pragma unroll
     for (int b = 0; b < BPLL; ++b)
 #pragma unroll
@@ -582,11 +719,11 @@ __global__ void __launch_bounds__(XY<N>::kThreads) xyf_warp_kernel(PassArgs a, f
   const float2* src;
   long long row_stride;
   if (XPASS) {
-    src = static_cast<const float2*>(a.g1) + g.g1_off + (long long)(it.u + r - 1) * r + it.v0;
-    row_stride = (long long)w * r;
+    src = static_cast<const float2*>(a.g1) + g.g1_off + (long long)(it.u + r - 1) * g.rp + it.v0;
+    row_stride = (long long)w * g.rp;
   } else {
-    src = static_cast<const float2*>(a.g2) + g.g2_off + (long long)it.u * N * r + it.v0;
-    row_stride = r;
+    src = static_cast<const float2*>(a.g2) + g.g2_off + (long long)it.u * N * g.rp + it.v0;
+    row_stride = g.rp;
   }
   for (int idx = tid; idx < N * kLines; idx += NT) {
     const int l = idx & (kLines - 1);
@@ -637,12 +774,12 @@ __global__ void __launch_bounds__(XY<N>::kThreads) xyf_warp_kernel(PassArgs a, f
       }
     }
   } else {
-    float2* dst = static_cast<float2*>(a.g1) + g.g1_off + (long long)it.u * w * r + it.v0;
+    float2* dst = static_cast<float2*>(a.g1) + g.g1_off + (long long)it.u * w * g.rp + it.v0;
     for (int idx = tid; idx < w * kLines; idx += NT) {
       const int l = idx & (kLines - 1);
       const int row = idx >> 3;
       const int ky = row - (r - 1);
-      if (l < it.cnt) dst[(long long)row * r + l] = bufs[(size_t)l * kBufLd + padn<N>(ky < 0 ? ky + N : ky)];
+      if (l < it.cnt) dst[(long long)row * g.rp + l] = bufs[(size_t)l * kBufLd + padn<N>(ky < 0 ? ky + N : ky)];
     }
   }
 }
@@ -676,6 +813,20 @@ bsp_status launch_zf(const PassArgs& a, const float* gfield, long long n_lines, 
 template <int N, bool XPASS>
 bsp_status launch_xy(const PassArgs& a, int n_items, int n_sm, cudaStream_t s) {
   if (n_items == 0) return BSP_OK;
+  if constexpr (xy_in_lines(N, XPASS)) {
+    const size_t smem = XYL<N>::kSmem;
+    auto kern = xy_line_kernel<N, XPASS>;
+    BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, XYL<N>::kThreads, smem));
+    constexpr int kUnits = XYL<N>::kThreads / 32;  // units of 4 lines a block takes at a time
+    const long long need = (2LL * n_items + kUnits - 1) / kUnits;
+    long long blocks = std::min<long long>((long long)std::max(per_sm, 1) * std::max(n_sm, 1), need);
+    if (!XPASS && a.grid_blocks > 0) blocks = std::min<long long>(a.grid_blocks, need);
+    kern<<<(unsigned)blocks, XYL<N>::kThreads, smem, s>>>(a, n_items);
+    BSP_CUDA(cudaGetLastError());
+    return BSP_OK;
+  } else {
   // two regions, each holding a tile of 2 r - 1 rows of the largest shell or, once it is read,
   // the line buffers
   const size_t smem = ((size_t)N + 2 * (size_t)xy_region<N>(a.rmax)) * sizeof(float2);
@@ -687,6 +838,7 @@ bsp_status launch_xy(const PassArgs& a, int n_items, int n_sm, cudaStream_t s) {
   xy_warp_kernel<N, XPASS><<<(unsigned)blocks, XY<N>::kThreads, smem, s>>>(a, n_items);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;
+  }
 }
 
 template <int S>

@@ -728,16 +728,16 @@ bsp_status host_plan(bsp_plan* p, const bsp_plan_desc* d) {
     g.qlo = (int)p->q[n];
     g.qhi = (int)p->q[n + 1];
     g.r = (int)isqrt_ll(p->q[n + 1] - 1) + 1;
-    g.pad = 0;
+    g.rp = row_pitch(g.r);
     g.g1_off = o1;
     g.g2_off = o2;
     if (p->dim == 2) {  // one buffer of X-pass rows [x][k_y < r], read again by the C2R along y
       g.g2_off = o1;
-      o1 += (long long)p->ngs * g.r;
+      o1 += (long long)p->ngs * g.rp;
       continue;
     }
-    o1 += (long long)p->ngs * (2 * g.r - 1) * g.r;
-    o2 += (long long)p->ngs * p->ngs * g.r;
+    o1 += (long long)p->ngs * (2 * g.r - 1) * g.rp;
+    o2 += (long long)p->ngs * p->ngs * g.rp;
   }
   // memory budget: stream x-slabs of the evaluation grid when all fields do not fit
   p->mem_budget = d->mem_budget_bytes;
@@ -768,13 +768,13 @@ void slab_items(int slab_nx, int grid, std::vector<Item>& zi, std::vector<int>& 
 
 long long g1_elems(const bsp_plan* p) {
   const ShellGeom& g = p->geom.back();
-  if (p->dim == 2) return g.g1_off + (long long)p->ngs * g.r;  // 2D X-pass rows [x][k_y < r]
-  return g.g1_off + (long long)p->ngs * (2 * g.r - 1) * g.r;
+  if (p->dim == 2) return g.g1_off + (long long)p->ngs * g.rp;  // 2D X-pass rows [x][k_y < r]
+  return g.g1_off + (long long)p->ngs * (2 * g.r - 1) * g.rp;
 }
 long long g2_elems(const bsp_plan* p) {
   const ShellGeom& g = p->geom.back();
   if (p->dim == 2) return 1;  // unused by 2D plans
-  return g.g2_off + (long long)p->ngs * p->ngs * g.r;
+  return g.g2_off + (long long)p->ngs * p->ngs * g.rp;
 }
 
 // Contraction autotuner (plans created with autotune = 1): for every tensor-core level, time its

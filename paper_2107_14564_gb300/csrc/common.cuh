@@ -54,10 +54,13 @@ struct Item { int n, u, v0, cnt; };
 struct ShellGeom {
   int qlo, qhi;        // modes with qlo <= |m|^2 < qhi
   int r;               // |m_i| <= r - 1 for every mode of the shell
-  int pad;
-  long long g1_off;    // complex offset of this shell in the X-pass buffer [x][2r-1][r]
-  long long g2_off;    // complex offset in the Y-pass buffer [x][y][r]
+  int rp;              // elements of a row of r k_z in the pass buffers (row_pitch(r))
+  long long g1_off;    // complex offset of this shell in the X-pass buffer [x][2r-1][rp]
+  long long g2_off;    // complex offset in the Y-pass buffer [x][y][rp]
 };
+// Rows of k_z start on 64-byte boundaries (FP32): the 8 (4) lines a block (warp) of the X and Y passes
+// moves at a time fill whole 32-byte sectors.
+inline int row_pitch(int r) { return (r + 7) / 8 * 8; }
 
 struct PassArgs {
   const void* spec;       // half spectrum (complex T), or null for the unit counting input
