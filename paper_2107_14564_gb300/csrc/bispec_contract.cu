@@ -8,7 +8,9 @@
 // FP32: an output's products are added in voxel order over runs of kSumRun voxels, the runs in
 // FP64. A lane owns one run and a warp one tile of 2 x 4 x 8 outputs (a, b, c), so 32 runs go
 // through the same 8 pair products and 64 multiply-adds per voxel and no lane idles for want of bins;
-// tiles at the edge of the triangle region take 2 b or 4 c.
+// tiles at the edge of the triangle region take 4 c. One block of 12 warps an SM (8 warps: 1.34 ms
+// per estimate at Ng = 256 and 24 shells, 12: 1.30, 16, which leaves 128 registers: 1.62; blocks of
+// tiles of 2 b as well were shorter and fewer fitted one block: 1.33 with 12).
 //   * What bounds it: the FMA units (at most 67% of their rate with three register reads each,
 //     measured on an outer product), then the warps' waits at the stages' barriers. Shared memory
 //     delivers 32 words per cycle whatever lanes share (measured: LDS.128 takes 4 cycles a warp even
@@ -106,23 +108,23 @@ __device__ __forceinline__ void lds_quad(uint32_t addr, float (&v)[4]) {
 
 // One quad of a tile whose fields are in registers: two neighbouring voxels' pair products are one
 // packed multiplication; their triple products are added in voxel order.
-template <int NB, int NC>
-__device__ __forceinline__ void sum_quad(const float (&a)[2][4], const float (&b)[NB][4], const float (&c)[NC][4],
+template <int NC>
+__device__ __forceinline__ void sum_quad(const float (&a)[2][4], const float (&b)[4][4], const float (&c)[NC][4],
                                          float (&acc)[64]) {
 #pragma unroll
   for (int h = 0; h < 4; h += 2) {
-    uint64_t p[2][NB];
+    uint64_t p[2][4];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int j = 0; j < NB; ++j)
+      for (int j = 0; j < 4; ++j)
         p[i][j] = ptx::f2_mul(ptx::f2_pack(a[i][h], a[i][h + 1]), ptx::f2_pack(b[j][h], b[j][h + 1]));
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
+        for (int j = 0; j < 4; ++j) {
           const float x = __uint_as_float((uint32_t)(e ? p[i][j] >> 32 : p[i][j]));
 #pragma unroll
           for (int k = 0; k < NC; ++k) acc[32 * i + 8 * j + k] = fmaf(x, c[k][h + e], acc[32 * i + 8 * j + k]);
@@ -133,24 +135,24 @@ __device__ __forceinline__ void sum_quad(const float (&a)[2][4], const float (&b
 // A stage, two quads at a time: the second's loads are under way while the first is summed. A, B, C
 // are the shared-memory addresses of this lane's row of the tile's fields, swz the exchange of its
 // quads (see contract_f32_kernel).
-template <int NB, int NC>
+template <int NC>
 __device__ __forceinline__ void sum_stage(const uint32_t (&A)[2], const uint32_t (&B)[4], const uint32_t (&C)[8],
                                           uint32_t off, uint32_t swz, float (&acc)[64]) {
 #pragma unroll 1
   for (uint32_t q = 0; q < kSumVox * 4; q += 32) {
-    float a[2][2][4], b[2][NB][4], c[2][NC][4];
+    float a[2][2][4], b[2][4][4], c[2][NC][4];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       const uint32_t o = off + ((q + 16 * t) ^ swz);
 #pragma unroll
       for (int i = 0; i < 2; ++i) lds_quad(A[i] + o, a[t][i]);
 #pragma unroll
-      for (int i = 0; i < NB; ++i) lds_quad(B[i] + o, b[t][i]);
+      for (int i = 0; i < 4; ++i) lds_quad(B[i] + o, b[t][i]);
 #pragma unroll
       for (int i = 0; i < NC; ++i) lds_quad(C[i] + o, c[t][i]);
     }
-    sum_quad<NB, NC>(a[0], b[0], c[0], acc);
-    sum_quad<NB, NC>(a[1], b[1], c[1], acc);
+    sum_quad<NC>(a[0], b[0], c[0], acc);
+    sum_quad<NC>(a[1], b[1], c[1], acc);
   }
 }
 
@@ -187,36 +189,45 @@ __global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a)
     runs[tid] = v;
   }
   __syncthreads();
-  // copies: this thread takes quad cq of run cr of every (kSumThreads / 32 kSumQuads)-th field
+  // copies: this thread takes quad cq of runs cr and cr + 16 of every (kSumThreads / 128)-th field
   const int stage_bytes = sub.nf * kSumFieldBytes;
-  const int cq = tid % kSumQuads, cr = (tid / kSumQuads) & 31;
-  constexpr int kStep = kSumThreads / (32 * kSumQuads);
-  static_assert(kStep >= 1 && kStep * 32 * kSumQuads == kSumThreads, "a thread copies one quad of one run");
-  const int f0 = tid / (32 * kSumQuads);
-  const int2 run = runs[cr];
+  const int cq = tid % kSumQuads, cr = (tid / kSumQuads) & 15;
+  constexpr int kStep = kSumThreads / (16 * kSumQuads);
+  static_assert(kStep >= 1 && kStep * 16 * kSumQuads == kSumThreads, "a thread copies one quad of two runs");
+  const int f0 = tid / (16 * kSumQuads);
+  const int2 run0 = runs[cr], run1 = runs[cr + 16];
 
   unsigned char* const cdst = smem + cr * kSumRow + ((cq ^ sum_swz(cr)) << 4);
+  static_assert(sum_swz(0) == sum_swz(16), "runs 16 apart exchange quads alike");
   auto issue = [&](int k, int buf) {
     unsigned char* dst = cdst + buf * stage_bytes;
-    const int v = run.x + k * kSumVox + 4 * cq;
-    const bool in = v < run.y;
+    const int v0 = run0.x + k * kSumVox + 4 * cq, v1 = run1.x + k * kSumVox + 4 * cq;
+    const bool in0 = v0 < run0.y, in1 = v1 < run1.y;
     if (L.t == 1) {
-      const float* src = fields + (in ? v : 0);
-      const uint32_t n = in ? 16u : 0u;
-#pragma unroll 4
-      for (int f = f0; f < sub.nf; f += kStep) ptx::cp_async16_zfill(dst + f * kSumFieldBytes, src + foff[f], n);
+      const float *src0 = fields + (in0 ? v0 : 0), *src1 = fields + (in1 ? v1 : 0);
+      const uint32_t n0 = in0 ? 16u : 0u, n1 = in1 ? 16u : 0u;
+#pragma unroll 2
+      for (int f = f0; f < sub.nf; f += kStep) {
+        const long long o = foff[f];
+        ptx::cp_async16_zfill(dst + f * kSumFieldBytes, src0 + o, n0);
+        ptx::cp_async16_zfill(dst + f * kSumFieldBytes + 16 * kSumRow, src1 + o, n1);
+      }
     } else {
-      long long o = 0;
-      if (in) {  // g is a multiple of 8: the quad lies in one row of the level's grid
+      auto at = [&](int v) {  // g is a multiple of 8: the quad lies in one row of the level's grid
         const unsigned g = (unsigned)L.g, u = (unsigned)v;
         const unsigned xy = u / g, z = u - xy * g, x = xy / g, y = xy - x * g;
-        o = ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
-      }
-      const float* src = fields + o;
-      for (int f = f0; f < sub.nf; f += kStep)
+        return ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
+      };
+      const float *src0 = fields + (in0 ? at(v0) : 0), *src1 = fields + (in1 ? at(v1) : 0);
+      for (int f = f0; f < sub.nf; f += kStep) {
+        const long long o = foff[f];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 4 * e, in ? src + foff[f] + e * L.t : fields, in ? 4u : 0u);
+        for (int e = 0; e < 4; ++e) {
+          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 4 * e, in0 ? src0 + o + e * L.t : fields, in0 ? 4u : 0u);
+          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 16 * kSumRow + 4 * e, in1 ? src1 + o + e * L.t : fields,
+                                 in1 ? 4u : 0u);
+        }
+      }
     }
     ptx::cp_async_commit();
   };
@@ -245,12 +256,8 @@ __global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a)
     if (k + 1 < nst) issue(k + 1, (k + 1) & 1);
     if (active) {
       const uint32_t off = (uint32_t)((k & 1) * stage_bytes);
-      switch (sub.kind) {  // the same for the block's tiles
-        case 3: sum_stage<4, 8>(A, B, C, off, swz, acc); break;
-        case 2: sum_stage<4, 4>(A, B, C, off, swz, acc); break;
-        case 1: sum_stage<2, 8>(A, B, C, off, swz, acc); break;
-        default: sum_stage<2, 4>(A, B, C, off, swz, acc);
-      }
+      if (sub.nc == 8) sum_stage<8>(A, B, C, off, swz, acc);
+      else sum_stage<4>(A, B, C, off, swz, acc);
     }
   }
   if (active) {

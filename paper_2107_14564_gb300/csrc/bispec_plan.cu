@@ -122,9 +122,9 @@ static int count_pair_quads(const std::vector<int>& ta, const std::vector<int>& 
 }
 
 // FP32 tables of a CUDA-core contraction level: tiles of 2 a x 4 (2) b x 8 (4) c taken off the bins from
-// the largest shells down, then blocks of `per` tiles of one kind that share fields, with the
+// the largest shells down, then blocks of `per` equally wide tiles that share fields, with the
 // fields they read. out[64 t + 32 i + 8 j + k]: the bin of output (i, j, k) of tile t.
-struct SumRaw { int a[2], b[4], c[8], kind, out[64]; };
+struct SumRaw { int a[2], b[4], c[8], nc, out[64]; };
 static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std::vector<int>& tb,
                                           const std::vector<int>& tc, const std::vector<int>* ids, int ncmax) {
   std::vector<SumRaw> raw;
@@ -164,7 +164,7 @@ static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std:
         for (int k = 0; k < 2; ++k) t.a[k] = as[i + (k < na ? k : 0)];
         for (size_t k = 0; k < 4; ++k) t.b[k] = ub[k < ub.size() ? k : 0];
         for (size_t k = 0; k < 8; ++k) t.c[k] = cs[m + (k < nc ? k : 0)];
-        t.kind = (ub.size() > 2 ? 2 : 0) + (nc > 4 ? 1 : 0);
+        t.nc = nc > 4 ? 8 : 4;
         for (int& o : t.out) o = -1;
         for (const B& x : rows)
           for (int ia = 0; ia < na; ++ia)
@@ -175,14 +175,14 @@ static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std:
       }
     }
   }
-  std::stable_sort(raw.begin(), raw.end(), [](const SumRaw& x, const SumRaw& y) { return x.kind > y.kind; });
+  std::stable_sort(raw.begin(), raw.end(), [](const SumRaw& x, const SumRaw& y) { return x.nc > y.nc; });
   return raw;
 }
 
 static void make_sum_subs(std::vector<SumRaw> raw, int per, std::vector<SumTile>& tiles, std::vector<SumSub>& subs,
                           std::vector<int>& sub_fields, std::vector<int>& map) {
-  while (!raw.empty()) {  // the first tile left, then those of its kind that add the fewest fields
-    SumSub sub{(int)tiles.size(), 0, (int)sub_fields.size(), 0, raw.front().kind};
+  while (!raw.empty()) {  // the first tile left, then those as wide that add the fewest fields
+    SumSub sub{(int)tiles.size(), 0, (int)sub_fields.size(), 0, raw.front().nc};
     std::vector<int> cur;
     auto with = [&](const SumRaw& t) {
       std::vector<int> u = cur;
@@ -197,7 +197,7 @@ static void make_sum_subs(std::vector<SumRaw> raw, int per, std::vector<SumTile>
     };
     while (sub.ntiles < per && !raw.empty()) {
       size_t best = 0, best_n = (size_t)-1;
-      for (size_t k = 0; k < raw.size() && raw[k].kind == sub.kind; ++k) {
+      for (size_t k = 0; k < raw.size() && raw[k].nc == sub.nc; ++k) {
         const size_t n = with(raw[k]).size();
         if (n < best_n) { best = k; best_n = n; }
         if (cur.empty()) break;
@@ -278,7 +278,7 @@ bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::ve
     const int gy = std::max((count_pair_quads(ta, tb, tc) + 255) / 256, 1);
     l.nblk_cap = (int)std::min<long long>(std::max(4 * p->n_sm / gy, 1), (nvox + 63) / 64);
     divide_sum_level(&l, nvox, 1, false);
-    // 8 c a tile; 4 (more tiles, each about half as long) on levels too small to give every SM 8;
+    // 8 c a tile; 4 (more tiles, each about half as long) on levels too small to fill every SM's warps;
     // then as many tiles a block as give every SM one
     std::vector<SumRaw> raw = make_sum_tiles(ta, tb, tc, ids, 8);
     if ((long long)raw.size() * l.splits < (long long)kSumWarps * p->n_sm) raw = make_sum_tiles(ta, tb, tc, ids, 4);

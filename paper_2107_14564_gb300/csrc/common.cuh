@@ -118,15 +118,15 @@ bsp_status launch_warp_yfpass(const PassArgs& a, int n_items, cudaStream_t s);
 bsp_status launch_warp_xfpass(const PassArgs& a, int n_items, float scale, cudaStream_t s);
 
 // ---------------------------------------------------------------- CUDA-core contraction tables
-// FP32: a tile is 2 x (4 or 2) x (8 or 4) outputs (a, b, c), one warp's registers; a sub is the up to
-// kSumWarps tiles of one block, of one kind (2 [4 b] + [8 c]), and the fields it stages; tiles name
-// fields by their place in that list. FP64: a job is one pair and n <= 4 third fields: f = (a, b, c0
+// FP32: a tile is 2 x 4 x (8 or 4) outputs (a, b, c), one warp's registers; a sub is the up to
+// kSumWarps tiles of one block, all nc = 8 or 4 wide, and the fields it stages; tiles name fields by
+// their place in that list. FP64: a job is one pair and n <= 4 third fields: f = (a, b, c0
 // .. c3).
 struct SumTile { uint8_t a[2], b[4], c[8], pad[2]; };
-struct SumSub { int tile0, ntiles, field0, nf, kind; };
+struct SumSub { int tile0, ntiles, field0, nf, nc; };
 struct SumJob { int f[6], n, pad; };
 
-constexpr int kSumWarps = 8;      // warps (tiles) of an FP32 block
+constexpr int kSumWarps = 12;     // warps (tiles) of an FP32 block
 constexpr int kSumMaxFields = 27; // fields an FP32 block stages at most (a tile has up to 14)
 constexpr int kSumRuns = 32;      // runs of an FP32 block, one per lane
 constexpr int kSumRun = 1024;     // voxels of one FP32 accumulation run
