@@ -160,7 +160,8 @@ __device__ __forceinline__ void sum_stage(const uint32_t (&A)[2], const uint32_t
 // for the sub's fields, [field][run][voxel], the quads of a run exchanged so that eight lanes' 16-byte
 // reads of one field meet all banks. 128 bytes a run and stage: a copy that brings less than a
 // cache line still occupies shared memory for a cycle (8 voxels a stage: 1.45 ms, 16: 1.25, 32:
-// 1.13, at Ng = 256 and 24 shells). One block of 8 warps an SM, two stages of up to 27 fields.
+// 1.13, at Ng = 256 and 24 shells). One block an SM, two stages of up to 27 fields (12 warps: 0.95 ms).
+// Copies go two runs a thread per look at a field's offset: 1.37 -> 1.30 ms per estimate, with 12 warps.
 __global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ long long foff[kSumMaxFields];
@@ -294,8 +295,10 @@ __global__ void __launch_bounds__(32 * kF64Warps, 4) contract_f64_kernel(SumArgs
   }
   __syncwarp();
   // Sums of kF64Run steps are added over the warp before they join the total: a lane that meets the
-  // counting fields' peak at the origin would otherwise round every later addition at its size.
-  double total = 0.0;
+  // counting fields' peak at the origin would otherwise round every later addition at its size. The
+  // total keeps its additions' rounding errors: at Ng = 768 and 24 shells a warp adds 1600 such sums,
+  // and what those after the peak lost to rounding, all the same way, moved a count off its integer.
+  double total = 0.0, lost = 0.0;
   const long long v0 = (long long)split * L.spw * 32;
   for (int k0 = 0; k0 < L.spw; k0 += kF64Run) {
     double acc[4 * kSumJobs];
@@ -326,10 +329,12 @@ __global__ void __launch_bounds__(32 * kF64Warps, 4) contract_f64_kernel(SumArgs
         if (n > 3) acc[4 * j + 3] = fma(p, d3, acc[4 * j + 3]);
       }
     }
-    total += warp_transpose_sum(acc, lane);
+    const double x = warp_transpose_sum(acc, lane), t = total + x, y = t - total;
+    lost += (total - (t - y)) + (x - y);
+    total = t;
   }
   const int e = set * 4 * kSumJobs + lane;
-  if (e < L.n_ent) L.partial[(long long)split * L.n_ent + e] = total;
+  if (e < L.n_ent) L.partial[(long long)split * L.n_ent + e] = total + lost;
 }
 
 // msum[map[e]] = scale * sum over the splits of partial[.][e] (added to msum when accumulating
