@@ -438,7 +438,7 @@ def run_ours(args, w):
         sm_mhz = pk.get("sm_max_mhz", 2070.0)
         alu_peak = 152 * 128 * 2 * sm_mhz * 1e6 / 1e12
         ach = wf[dom] / tdom / 1e12
-        roof = {"bound": "alu", "kernel": "contract_simt_kernel<float>", "achieved": round(ach, 2),
+        roof = {"bound": "alu", "kernel": "contract_f32_kernel", "achieved": round(ach, 2),
                 "peak": round(alu_peak, 1), "unit": "TFLOP/s", "frac": round(ach / alu_peak, 4),
                 "peak_kind": f"FP32 CUDA-core FMA, 152 SM x 128 lanes x 2 x {sm_mhz:.0f} MHz",
                 "traffic": ncu_traffic(dname, args.workload, args.precision)}

@@ -19,13 +19,15 @@
 //   * loader warp: per 64-voxel chunk, two tiled TMA loads (high and low plane) bring NP shell
 //     rows of 128 bytes with the 128-byte swizzle into an NB-stage shared-memory ring; they
 //     complete on the stage's "full" mbarrier. The same bytes are the B operand of the MMAs.
-//   * 16 generator warps (4 per TMEM lane quarter: 2 lane halves x 2 K-step pairs): a quad of
+//   * 16 generator warps (4 per TMEM lane quarter: 2 lane halves x 2 alternating chunks): a quad of
 //     threads owns one slot, rows r (Ph) and r + 8 (Pl) of a 16-lane half, each thread four
 //     voxels of every K step. It loads its slot's fields from shared memory, forms the products
 //     in bf16x2 arithmetic and writes them into the tensor-memory A stage of each tile with
 //     tcgen05.st .16x256b (whose lane map puts a thread's registers in rows r and r + 8). A warp
-//     hands chunk i - 1's stage over while chunk i's loads are in flight, forms chunk i's
-//     products and only then waits for the MMAs of chunk i - NA to free its A stage.
+//     takes every other chunk whole (all 4 K steps): it hands its last chunk's stage over while
+//     this chunk's loads are in flight, forms the products and only then waits for the MMAs of
+//     chunk i - NA to free its A stage. Half of each chunk per warp instead paid the stage
+//     hand-over and the waits twice as often (3.39 -> 3.35 ms at Ng = 512 and 32 shells).
 //   * KT MMA warps, one per tile: one thread issues the tile's 4 MMAs of a chunk into its FP32
 //     accumulator and commits them to the B stage's "mma done" mbarrier (KT arrivals), which frees
 //     the B stage for the loader and (NA chunks later) the A stage for the generators. One

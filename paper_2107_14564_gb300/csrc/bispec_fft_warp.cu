@@ -1,16 +1,16 @@
-// Warp-per-line shell FFT passes for FP32 plans whose grid side is a power of two (128..1024).
+// Warp-per-line shell FFT passes for FP32 plans on grids of 2^p or 3 2^p points a side (128..1024).
 //
 // Same three passes as the generic kernels (X and Y: C2C of the lines that meet each shell's
 // ball; Z: C2R of the r_n leading k_z values into the real shell field d_n, Eq. (2.8)), but every
-// line is transformed by one warp with all index arithmetic fixed at compile time:
-//   * a lane holds N/32 points of the line in registers; a Stockham stage of radix R runs
-//     N/(32 R) butterflies per lane, and between stages the warp exchanges its points through
+// line is transformed by 8 to 32 lanes of a warp with all index arithmetic fixed at compile time:
+//   * a lane holds N/LPL points of the line in registers; a Stockham stage of radix R runs
+//     N/(LPL R) butterflies per lane, and between stages the lanes exchange their points through
 //     its own padded shared-memory buffer (one __syncwarp, no block barrier);
-//   * the first stage reads x[j + r N/R] and the last writes y[j + r N/R], j = lane + 32 b, so a
+//   * the first stage reads x[j + r N/R] and the last writes y[j + r N/R], j = lane + LPL b, so a
 //     warp's global loads and stores are contiguous along the line;
-//   * X and Y passes stage a [2r_n - 1][16] tile of their input (16 lines, contiguous along k_z)
-//     and a [N][16] tile of their output in shared memory, so global traffic stays coalesced
-//     even though their lines run along the slow axes;
+//   * X (to 256 points) and Y (to 384) passes take 4 neighbouring k_z a warp, 8 lanes a line, and go
+//     from global memory to registers and back (xy_line_kernel); longer lines stage a tile of 8
+//     lines in shared memory, so global traffic stays coalesced although lines run along slow axes;
 //   * the Z pass forms the half-length input Z[k] = (X[k] + conj X[M-k]) + i (X[k] - conj X[M-k])
 //     W^k directly from global memory and writes z[n] = x[2n] + i x[2n+1] straight to the field.
 #include "common.cuh"
