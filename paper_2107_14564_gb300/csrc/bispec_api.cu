@@ -118,7 +118,7 @@ bsp_status contract_slab(bsp_plan* p, int k, cudaStream_t s) {
     if (st != BSP_OK) return st;
     return launch_reduce_tc_all(p->d_tc_bins, (int)p->trips.size(), p->msum, s, k > 0);
   }
-  SumArgs a = last ? p->sums_last : p->sums;
+  SumArgs a = last ? p->sums_last : p->sums_slab;
   a.fields = p->fields;
   a.msum = p->msum;
   a.accumulate = k > 0;
@@ -282,7 +282,7 @@ bsp_status estimate_impl(bsp_plan* p, const void* spec, double* b_trip, double* 
       int passes = p->warp_fft ? 2 + p->n_slabs() : (p->nxi > 0) + (p->nyi > 0);
       if (!p->warp_fft)
         for (int k = 0; k < p->n_slabs(); ++k) passes += p->zi_off[k + 1] > p->zi_off[k];
-      const bool work = !p->levels.empty() && (split ? p->levels[0].n_tg > 0 : p->sums.items > 0);
+      const bool work = !p->levels.empty() && (split ? p->levels[0].n_tg > 0 : p->sums_slab.items > 0);
       p->launches += passes + 2LL * work * p->n_slabs() + 1;
     } else {
       const int passes = (p->warp_fft ? 3 : (p->nxi > 0) + (p->nyi > 0) + (p->nzi > 0) + (split ? 1 : 0)) +

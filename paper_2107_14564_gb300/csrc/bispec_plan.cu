@@ -305,7 +305,7 @@ bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::ve
   return BSP_OK;
 }
 
-bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel> lv, const std::vector<long long>& nvox, int spw, bool f64,
+bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel>& lv, const std::vector<long long>& nvox, int spw, bool f64,
                          SumArgs* out, std::vector<void*>* owned, cudaStream_t s) {
   SumArgs a{};
   bsp_status st;
@@ -317,10 +317,12 @@ bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel> lv, const std::vecto
     a.items += l.units * l.splits;
     a.n_ent += l.n_ent;
     if (!f64) a.smem = std::max(a.smem, sum_stage_bytes(l.max_nf));
+    if (l.splits <= l.rows) continue;  // the partial sums of an earlier division of this level
     void* d = nullptr;
     if ((st = dev_alloc(p, (size_t)l.splits * l.n_ent * sizeof(double), &d)) != BSP_OK) return st;
     if (owned) owned->push_back(d);
     l.partial = static_cast<double*>(d);
+    l.rows = l.splits;
   }
   SumLevel* d = nullptr;
   if ((st = dev_upload(p, lv, &d, s)) != BSP_OK) return st;
@@ -949,13 +951,14 @@ void merge_tc_levels(const bsp_plan* p, std::vector<std::pair<int, std::vector<i
   }
 }
 
-// The CUDA-core contraction launches of the plan: every level at once, largest first; a plan
-// streaming x-slabs has one level and two slab lengths.
+// The CUDA-core contraction launches of the plan: every level at once, largest first. A plan streaming
+// x-slabs has one level and three launches of it: a full slab's, the last slab's, and the whole
+// grid's for bsp_contract, whose caller holds every voxel. They share their partial sums, since a plan's
+// calls run one after the other.
 bsp_status build_sums(bsp_plan* p, cudaStream_t s) {
   const bool f64 = p->prec == BSP_FP64;
-  const int last = p->n_slabs() - 1;
   std::vector<SumLevel> lv;
-  std::vector<long long> nvox[2];
+  std::vector<long long> whole;  // voxels of each level
   bsp_status st;
   for (size_t i = p->levels.size(); i-- > 0;) {
     const ContractLevel& L = p->levels[i];
@@ -971,23 +974,26 @@ bsp_status build_sums(bsp_plan* p, cudaStream_t s) {
     l.t = L.stride;
     l.s = p->ngs;
     l.scale = L.scale;
-    const long long n0 = p->slab_nx ? (long long)p->slab_len(0) * p->ngs * p->ngs : L.nvox();
-    const long long n1 = p->slab_nx ? (long long)p->slab_len(last) * p->ngs * p->ngs : n0;
-    st = make_sum_level(p, ta, tb, tc, &L.bins, f64, p->slab_nx ? p->nvox() : n0, &l, nullptr, s);
-    if (st != BSP_OK) return st;
+    if ((st = make_sum_level(p, ta, tb, tc, &L.bins, f64, L.nvox(), &l, nullptr, s)) != BSP_OK) return st;
     lv.push_back(l);
-    nvox[0].push_back(n0);
-    nvox[1].push_back(n1);
+    whole.push_back(L.nvox());
   }
-  long long steps = 0;
-  for (size_t i = 0; i < lv.size(); ++i) steps += (nvox[0][i] + 31) / 32 * lv[i].units;
-  const int spw = sum_steps_per_warp(steps, p->n_sm);
-  for (int k = 0; k < 2; ++k) {
-    for (size_t i = 0; i < lv.size(); ++i) lv[i].fstride = p->slab_nx ? nvox[k][i] : p->nvox();
-    if (k == 1 && nvox[1] == nvox[0]) p->sums_last = p->sums;
-    else if ((st = make_sum_args(p, lv, nvox[k], spw, f64, k ? &p->sums_last : &p->sums, nullptr, s)) != BSP_OK) return st;
-  }
-  return BSP_OK;
+  auto spw = [&](const std::vector<long long>& nvox) {
+    long long steps = 0;
+    for (size_t i = 0; i < lv.size(); ++i) steps += (nvox[i] + 31) / 32 * lv[i].units;
+    return sum_steps_per_warp(steps, p->n_sm);
+  };
+  for (SumLevel& l : lv) l.fstride = p->nvox();
+  if ((st = make_sum_args(p, lv, whole, spw(whole), f64, &p->sums, nullptr, s)) != BSP_OK) return st;
+  if (!p->slab_nx || lv.empty()) return BSP_OK;
+  auto slab = [&](int k, int steps, SumArgs* out) {
+    lv[0].fstride = (long long)p->slab_len(k) * p->ngs * p->ngs;
+    return make_sum_args(p, lv, {lv[0].fstride}, steps, f64, out, nullptr, s);
+  };
+  const int last = p->n_slabs() - 1, steps = spw({(long long)p->slab_len(0) * p->ngs * p->ngs});
+  if ((st = slab(0, steps, &p->sums_slab)) != BSP_OK) return st;
+  p->sums_last = p->sums_slab;
+  return p->slab_len(last) == p->slab_len(0) ? BSP_OK : slab(last, steps, &p->sums_last);
 }
 
 // Contraction levels (see ContractLevel): each pair (a, b) of the kept bins goes to the smallest

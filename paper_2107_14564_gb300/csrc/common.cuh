@@ -152,6 +152,7 @@ struct SumLevel {
   const int* map;          // [n_ent] bin of each output (64 per tile, 4 per job), -1: none
   int n_ent, ent0;         // outputs, first output of the level in the launch
   double* partial;         // [splits][n_ent]
+  int rows;                // splits that fit `partial`
   double scale;            // msum = scale * sum
 };
 struct SumArgs {

@@ -125,7 +125,8 @@ struct bsp_plan {
   int nwxi = 0, nwyi = 0;
   int rmax = 0;
   std::vector<ContractLevel> levels;
-  SumArgs sums{}, sums_last{};  // CUDA-core contraction of every level; of the last x-slab
+  // CUDA-core contraction of every level over the whole grid; with x-slabs, of a full slab and of the last
+  SumArgs sums{}, sums_slab{}, sums_last{};
   // each level's side and bins before split-BF16 plans merge levels (every pair on its smallest
   // exact grid): the algorithm's work, which bsp_plan_stage_work counts
   std::vector<std::pair<int, std::vector<int>>> exact_levels;
@@ -204,12 +205,13 @@ void make_items(const bsp_plan* p, const PassLines& lines, std::vector<Item>& xi
                 std::vector<Item>& yi, std::vector<Item>& zi);
 // Device tables of a CUDA-core contraction level over bins (a, b, c) sorted by (a, b, c), ids[i] (or i)
 // the output of bin i; the caller gives *l the sampling and the scale. make_sum_args divides the
-// levels' voxels over a launch and allocates its partial sums. Allocations are also appended to
-// `owned` if given.
+// levels' voxels over a launch and allocates its partial sums where those of an earlier division of lv
+// are too few: launches that share them run one after the other. Allocations are also appended
+// to `owned` if given.
 bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::vector<int>& tb,
                           const std::vector<int>& tc, const std::vector<int>* ids, bool f64, long long nvox,
                           SumLevel* l, std::vector<void*>* owned, cudaStream_t s);
-bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel> lv, const std::vector<long long>& nvox, int spw, bool f64,
+bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel>& lv, const std::vector<long long>& nvox, int spw, bool f64,
                          SumArgs* out, std::vector<void*>* owned, cudaStream_t s);
 // Pair groups of the tensor-core contraction of one level: the slots (f0, f1, f2, flags) of n_tg
 // tile groups of kt tiles, and where[i] = (tg * kt + j) * kTcSlots + slot for pair i.
