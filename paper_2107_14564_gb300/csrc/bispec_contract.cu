@@ -334,7 +334,8 @@ __global__ void __launch_bounds__(32 * kF64Warps, 4) contract_f64_kernel(SumArgs
     total = t;
   }
   const int e = set * 4 * kSumJobs + lane;
-  if (e < L.n_ent) L.partial[(long long)split * L.n_ent + e] = total + lost;
+  // once a total is infinite, the differences above are NaN: it has no rounding errors to add
+  if (e < L.n_ent) L.partial[(long long)split * L.n_ent + e] = isfinite(lost) ? total + lost : total;
 }
 
 // msum[map[e]] = scale * sum over the splits of partial[.][e] (added to msum when accumulating
