@@ -426,10 +426,10 @@ bsp_status grad_setup(bsp_plan* p, cudaStream_t s) {
     add(b.a, b.c, b.b, (int)t);
     add(b.a, b.b, b.c, (int)t);
   }
-  // the lists of launch_adjoint_products, each made even by a pair without bins
+  // the lists of launch_adjoint_products, each made even by its last pair once more, without bins (a
+  // product no bin needs may overflow, and 0 times it spoils every G_n of the list)
   std::vector<int2> pairs;
   std::vector<int> ptr(1, 0), idx;
-  const Pair none{make_int2(0, 0), 0, 0, std::vector<std::vector<int>>(np)};
   auto place = [&](const Pair& q) {
     pairs.push_back(q.ab);
     for (const std::vector<int>& b : q.bins) {
@@ -444,7 +444,7 @@ bsp_status grad_setup(bsp_plan* p, cudaStream_t s) {
       while (q.q0 < adj_range(first, np / 4).q0 || q.q1 > adj_range(first, np / 4).q1) ++first;
       if (first == k) place(q);
     }
-    if (pairs.size() % 2) place(none);
+    if (pairs.size() % 2) place({pairs.back(), 0, 0, std::vector<std::vector<int>>(np)});
   }
   p->adj_lists.p[kAdjRanges] = (int)pairs.size();
   p->adj_entries = (int)pairs.size() * np;
