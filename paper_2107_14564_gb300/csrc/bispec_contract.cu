@@ -156,7 +156,7 @@ __device__ __forceinline__ void sum_stage(const uint32_t (&A)[2], const uint32_t
   }
 }
 
-// Block = (level, sub, group of 32 runs). A stage holds kSumVox voxels of every run of the group
+// Block = (level, sub, gps groups of 32 runs). A stage holds kSumVox voxels of every run of the group
 // for the sub's fields, [field][run][voxel], the quads of a run exchanged so that eight lanes' 16-byte
 // reads of one field meet all banks. 128 bytes a run and stage: a copy that brings less than a
 // cache line still occupies shared memory for a cycle (8 voxels a stage: 1.45 ms, 16: 1.25, 32:
@@ -169,69 +169,18 @@ __global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a)
   const int lane = tid & 31;
   const SumLevel L = level_of(a, blockIdx.x);
   const int unit = (int)(blockIdx.x - L.w0);
-  const int grp = unit / L.units;  // the subs of a group run side by side: its fields stay in L2
-  const SumSub sub = L.subs[unit - grp * L.units];
+  const int split = unit / L.units;  // the subs of a group run side by side: its fields stay in L2
+  const SumSub sub = L.subs[unit - split * L.units];
   const float* fields = static_cast<const float*>(a.fields);
   if (tid < sub.nf) foff[tid] = (long long)L.sub_fields[sub.field0 + tid] * L.fstride;
-  // the runs of the group: whole runs first, then the summation blocks' remainders; lane r sums run r
-  const bool whole = grp < L.ngf;
-  const int len = whole ? kSumRun : L.vpb - L.nfull * kSumRun;
-  __shared__ int2 runs[32];
-  if (tid < 32) {
-    const int i = (whole ? grp : grp - L.ngf) * 32 + tid;
-    const int b = whole ? i / L.nfull : i;
-    int2 v = make_int2(0, 0);
-    if (b < L.nblk) {
-      const long long first = (long long)b * L.vpb;
-      const long long start = first + (long long)(whole ? i - b * L.nfull : L.nfull) * kSumRun;
-      const long long end = min(min(first + (long long)L.vpb, L.nvox), start + (long long)len);
-      if (end > start) v = make_int2((int)start, (int)end);
-    }
-    runs[tid] = v;
-  }
-  __syncthreads();
   // copies: this thread takes quad cq of runs cr and cr + 16 of every (kSumThreads / 128)-th field
   const int stage_bytes = sub.nf * kSumFieldBytes;
   const int cq = tid % kSumQuads, cr = (tid / kSumQuads) & 15;
   constexpr int kStep = kSumThreads / (16 * kSumQuads);
   static_assert(kStep >= 1 && kStep * 16 * kSumQuads == kSumThreads, "a thread copies one quad of two runs");
   const int f0 = tid / (16 * kSumQuads);
-  const int2 run0 = runs[cr], run1 = runs[cr + 16];
-
   unsigned char* const cdst = smem + cr * kSumRow + ((cq ^ sum_swz(cr)) << 4);
   static_assert(sum_swz(0) == sum_swz(16), "runs 16 apart exchange quads alike");
-  auto issue = [&](int k, int buf) {
-    unsigned char* dst = cdst + buf * stage_bytes;
-    const int v0 = run0.x + k * kSumVox + 4 * cq, v1 = run1.x + k * kSumVox + 4 * cq;
-    const bool in0 = v0 < run0.y, in1 = v1 < run1.y;
-    if (L.t == 1) {
-      const float *src0 = fields + (in0 ? v0 : 0), *src1 = fields + (in1 ? v1 : 0);
-      const uint32_t n0 = in0 ? 16u : 0u, n1 = in1 ? 16u : 0u;
-#pragma unroll 2
-      for (int f = f0; f < sub.nf; f += kStep) {
-        const long long o = foff[f];
-        ptx::cp_async16_zfill(dst + f * kSumFieldBytes, src0 + o, n0);
-        ptx::cp_async16_zfill(dst + f * kSumFieldBytes + 16 * kSumRow, src1 + o, n1);
-      }
-    } else {
-      auto at = [&](int v) {  // g is a multiple of 8: the quad lies in one row of the level's grid
-        const unsigned g = (unsigned)L.g, u = (unsigned)v;
-        const unsigned xy = u / g, z = u - xy * g, x = xy / g, y = xy - x * g;
-        return ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
-      };
-      const float *src0 = fields + (in0 ? at(v0) : 0), *src1 = fields + (in1 ? at(v1) : 0);
-      for (int f = f0; f < sub.nf; f += kStep) {
-        const long long o = foff[f];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 4 * e, in0 ? src0 + o + e * L.t : fields, in0 ? 4u : 0u);
-          ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 16 * kSumRow + 4 * e, in1 ? src1 + o + e * L.t : fields,
-                                 in1 ? 4u : 0u);
-        }
-      }
-    }
-    ptx::cp_async_commit();
-  };
   const int warp = tid >> 5;
   uint32_t A[2], B[4], C[8];
   const bool active = warp < sub.ntiles;
@@ -246,29 +195,85 @@ __global__ void __launch_bounds__(kSumThreads, 1) contract_f32_kernel(SumArgs a)
 #pragma unroll
     for (int i = 0; i < 8; ++i) C[i] = row + t.c[i] * kSumFieldBytes;
   }
-  float acc[64];
-#pragma unroll
-  for (int i = 0; i < 64; ++i) acc[i] = 0.f;
-  const int nst = len / kSumVox;
-  issue(0, 0);
-  for (int k = 0; k < nst; ++k) {
-    ptx::cp_async_wait<0>();  // stage k has landed
-    __syncthreads();          // for every thread, and stage k - 1 has been read
-    if (k + 1 < nst) issue(k + 1, (k + 1) & 1);
-    if (active) {
-      const uint32_t off = (uint32_t)((k & 1) * stage_bytes);
-      if (sub.nc == 8) sum_stage<8>(A, B, C, off, swz, acc);
-      else sum_stage<4>(A, B, C, off, swz, acc);
+  const int g0 = split * L.gps, g1 = min(g0 + L.gps, L.ngrp);
+#pragma unroll 1
+  for (int grp = g0; grp < g1; ++grp) {
+    // the runs of the group: whole runs first, then the summation blocks' remainders; lane r sums run r
+    const bool whole = grp < L.ngf;
+    const int len = whole ? kSumRun : L.vpb - L.nfull * kSumRun;
+    __shared__ int2 runs[32];
+    if (grp > g0) __syncthreads();  // the last group's runs and stages have been read
+    if (tid < 32) {
+      const int i = (whole ? grp : grp - L.ngf) * 32 + tid;
+      const int b = whole ? i / L.nfull : i;
+      int2 v = make_int2(0, 0);
+      if (b < L.nblk) {
+        const long long first = (long long)b * L.vpb;
+        const long long start = first + (long long)(whole ? i - b * L.nfull : L.nfull) * kSumRun;
+        const long long end = min(min(first + (long long)L.vpb, L.nvox), start + (long long)len);
+        if (end > start) v = make_int2((int)start, (int)end);
+      }
+      runs[tid] = v;
     }
-  }
-  if (active) {
-    float half[32];
+    __syncthreads();
+    const int2 run0 = runs[cr], run1 = runs[cr + 16];
+    auto issue = [&](int k, int buf) {
+      unsigned char* dst = cdst + buf * stage_bytes;
+      const int v0 = run0.x + k * kSumVox + 4 * cq, v1 = run1.x + k * kSumVox + 4 * cq;
+      const bool in0 = v0 < run0.y, in1 = v1 < run1.y;
+      if (L.t == 1) {
+        const float *src0 = fields + (in0 ? v0 : 0), *src1 = fields + (in1 ? v1 : 0);
+        const uint32_t n0 = in0 ? 16u : 0u, n1 = in1 ? 16u : 0u;
+#pragma unroll 2
+        for (int f = f0; f < sub.nf; f += kStep) {
+          const long long o = foff[f];
+          ptx::cp_async16_zfill(dst + f * kSumFieldBytes, src0 + o, n0);
+          ptx::cp_async16_zfill(dst + f * kSumFieldBytes + 16 * kSumRow, src1 + o, n1);
+        }
+      } else {
+        auto at = [&](int v) {  // g is a multiple of 8: the quad lies in one row of the level's grid
+          const unsigned g = (unsigned)L.g, u = (unsigned)v;
+          const unsigned xy = u / g, z = u - xy * g, x = xy / g, y = xy - x * g;
+          return ((long long)x * L.t * L.s + (long long)y * L.t) * L.s + (long long)z * L.t;
+        };
+        const float *src0 = fields + (in0 ? at(v0) : 0), *src1 = fields + (in1 ? at(v1) : 0);
+        for (int f = f0; f < sub.nf; f += kStep) {
+          const long long o = foff[f];
 #pragma unroll
-    for (int m = 0; m < 2; ++m) {
+          for (int e = 0; e < 4; ++e) {
+            ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 4 * e, in0 ? src0 + o + e * L.t : fields, in0 ? 4u : 0u);
+            ptx::cp_async_zfill<4>(dst + f * kSumFieldBytes + 16 * kSumRow + 4 * e, in1 ? src1 + o + e * L.t : fields,
+                                   in1 ? 4u : 0u);
+          }
+        }
+      }
+      ptx::cp_async_commit();
+    };
+    float acc[64];
 #pragma unroll
-      for (int i = 0; i < 32; ++i) half[i] = acc[32 * m + i];
-      const double s = warp_transpose_sum(half, lane);
-      L.partial[(long long)grp * L.n_ent + (sub.tile0 + warp) * 64 + 32 * m + lane] = s;
+    for (int i = 0; i < 64; ++i) acc[i] = 0.f;
+    const int nst = len / kSumVox;
+    issue(0, 0);
+    for (int k = 0; k < nst; ++k) {
+      ptx::cp_async_wait<0>();  // stage k has landed
+      __syncthreads();          // for every thread, and stage k - 1 has been read
+      if (k + 1 < nst) issue(k + 1, (k + 1) & 1);
+      if (active) {
+        const uint32_t off = (uint32_t)((k & 1) * stage_bytes);
+        if (sub.nc == 8) sum_stage<8>(A, B, C, off, swz, acc);
+        else sum_stage<4>(A, B, C, off, swz, acc);
+      }
+    }
+    if (active) {
+      float half[32];
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) half[i] = acc[32 * m + i];
+        const double s = warp_transpose_sum(half, lane);
+        double* out = L.partial + (long long)split * L.n_ent + (sub.tile0 + warp) * 64 + 32 * m + lane;
+        *out = grp > g0 ? *out + s : s;  // this lane's alone
+      }
     }
   }
 }

@@ -237,8 +237,9 @@ static void make_sum_jobs(const std::vector<int>& ta, const std::vector<int>& tb
 }
 
 // FP32: the summation blocks of `nvox` voxels (a multiple of 64 voxels each), their whole runs in
-// groups of kSumRuns and their remainders likewise. FP64: steps of 32 voxels, spw of them per warp.
-static void divide_sum_level(SumLevel* l, long long nvox, int spw, bool f64) {
+// groups of kSumRuns and their remainders likewise, as many groups a block as leave kSumWaves blocks
+// per SM. FP64: steps of 32 voxels, spw of them per warp.
+static void divide_sum_level(SumLevel* l, long long nvox, int spw, bool f64, int n_sm) {
   l->nvox = nvox;
   if (f64) {
     l->spw = spw;
@@ -250,7 +251,10 @@ static void divide_sum_level(SumLevel* l, long long nvox, int spw, bool f64) {
   l->nblk = (int)((nvox + l->vpb - 1) / l->vpb);
   l->nfull = l->vpb / kSumRun;
   l->ngf = (int)(((long long)l->nblk * l->nfull + kSumRuns - 1) / kSumRuns);
-  l->splits = l->ngf + (l->vpb % kSumRun ? (l->nblk + kSumRuns - 1) / kSumRuns : 0);
+  l->ngrp = l->ngf + (l->vpb % kSumRun ? (l->nblk + kSumRuns - 1) / kSumRuns : 0);
+  const long long most = (long long)kSumWaves * std::max(1, n_sm);
+  l->gps = (int)std::max<long long>(1, ((long long)l->ngrp * l->units + most - 1) / most);
+  l->splits = (l->ngrp + l->gps - 1) / l->gps;
 }
 
 bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::vector<int>& tb,
@@ -277,12 +281,12 @@ bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::ve
     // of 256 4 x 4 tiles
     const int gy = std::max((count_pair_quads(ta, tb, tc) + 255) / 256, 1);
     l.nblk_cap = (int)std::min<long long>(std::max(4 * p->n_sm / gy, 1), (nvox + 63) / 64);
-    divide_sum_level(&l, nvox, 1, false);
+    divide_sum_level(&l, nvox, 1, false, p->n_sm);
     // 8 c a tile; 4 (more tiles, each about half as long) on levels too small to fill every SM's warps;
     // then as many tiles a block as give every SM one
     std::vector<SumRaw> raw = make_sum_tiles(ta, tb, tc, ids, 8);
-    if ((long long)raw.size() * l.splits < (long long)kSumWarps * p->n_sm) raw = make_sum_tiles(ta, tb, tc, ids, 4);
-    const long long each = ((long long)raw.size() * l.splits + p->n_sm - 1) / p->n_sm;
+    if ((long long)raw.size() * l.ngrp < (long long)kSumWarps * p->n_sm) raw = make_sum_tiles(ta, tb, tc, ids, 4);
+    const long long each = ((long long)raw.size() * l.ngrp + p->n_sm - 1) / p->n_sm;
     const int per = (int)std::max<long long>(1, std::min<long long>(kSumWarps, each));
     std::vector<SumTile> tiles;
     std::vector<SumSub> subs;
@@ -311,18 +315,18 @@ bsp_status make_sum_args(bsp_plan* p, std::vector<SumLevel>& lv, const std::vect
   bsp_status st;
   for (size_t i = 0; i < lv.size(); ++i) {
     SumLevel& l = lv[i];
-    divide_sum_level(&l, nvox[i], spw, f64);
+    divide_sum_level(&l, nvox[i], spw, f64, p->n_sm);
     l.w0 = a.items;
     l.ent0 = a.n_ent;
     a.items += l.units * l.splits;
     a.n_ent += l.n_ent;
     if (!f64) a.smem = std::max(a.smem, sum_stage_bytes(l.max_nf));
-    if (l.splits <= l.rows) continue;  // the partial sums of an earlier division of this level
+    if (l.partial && l.splits <= l.rows) continue;  // the partial sums of an earlier division of this level
+    l.rows = std::max(l.rows, l.splits);
     void* d = nullptr;
-    if ((st = dev_alloc(p, (size_t)l.splits * l.n_ent * sizeof(double), &d)) != BSP_OK) return st;
+    if ((st = dev_alloc(p, (size_t)l.rows * l.n_ent * sizeof(double), &d)) != BSP_OK) return st;
     if (owned) owned->push_back(d);
     l.partial = static_cast<double*>(d);
-    l.rows = l.splits;
   }
   SumLevel* d = nullptr;
   if ((st = dev_upload(p, lv, &d, s)) != BSP_OK) return st;
@@ -983,17 +987,27 @@ bsp_status build_sums(bsp_plan* p, cudaStream_t s) {
     for (size_t i = 0; i < lv.size(); ++i) steps += (nvox[i] + 31) / 32 * lv[i].units;
     return sum_steps_per_warp(steps, p->n_sm);
   };
+  const int last = p->n_slabs() - 1;
+  auto slab_vox = [&](int k) { return (long long)p->slab_len(k) * p->ngs * p->ngs; };
+  int steps = 0;
+  if (p->slab_nx && !lv.empty()) {
+    steps = spw({slab_vox(0)});
+    for (int k : {0, last}) {  // rows for the slabs' divisions too
+      SumLevel l = lv[0];
+      divide_sum_level(&l, slab_vox(k), steps, f64, p->n_sm);
+      lv[0].rows = std::max(lv[0].rows, l.splits);
+    }
+  }
   for (SumLevel& l : lv) l.fstride = p->nvox();
   if ((st = make_sum_args(p, lv, whole, spw(whole), f64, &p->sums, nullptr, s)) != BSP_OK) return st;
   if (!p->slab_nx || lv.empty()) return BSP_OK;
-  auto slab = [&](int k, int steps, SumArgs* out) {
-    lv[0].fstride = (long long)p->slab_len(k) * p->ngs * p->ngs;
-    return make_sum_args(p, lv, {lv[0].fstride}, steps, f64, out, nullptr, s);
+  auto slab = [&](int k, SumArgs* out) {
+    lv[0].fstride = slab_vox(k);
+    return make_sum_args(p, lv, {slab_vox(k)}, steps, f64, out, nullptr, s);
   };
-  const int last = p->n_slabs() - 1, steps = spw({(long long)p->slab_len(0) * p->ngs * p->ngs});
-  if ((st = slab(0, steps, &p->sums_slab)) != BSP_OK) return st;
+  if ((st = slab(0, &p->sums_slab)) != BSP_OK) return st;
   p->sums_last = p->sums_slab;
-  return p->slab_len(last) == p->slab_len(0) ? BSP_OK : slab(last, steps, &p->sums_last);
+  return p->slab_len(last) == p->slab_len(0) ? BSP_OK : slab(last, &p->sums_last);
 }
 
 // Contraction levels (see ContractLevel): each pair (a, b) of the kept bins goes to the smallest

@@ -131,10 +131,14 @@ constexpr int kSumMaxFields = 27; // fields an FP32 block stages at most (a tile
 constexpr int kSumRuns = 32;      // runs of an FP32 block, one per lane
 constexpr int kSumRun = 1024;     // voxels of one FP32 accumulation run
 constexpr int kSumJobs = 8;       // FP64 jobs of a warp
+// FP32 blocks of a level per SM above which a block takes several groups: partial sums, one row a block,
+// stay within 64 x SMs x kSumWarps x 64 doubles (60 MB) whatever the voxels, and the last wave
+// within 1/32 of the time.
+constexpr int kSumWaves = 64;
 
 // One level of a CUDA-core contraction launch: triple sums over the g^3 voxels sampled from source
 // fields of side s with stride t (t == 1: over the nvox voxels as they lie in memory). Its work
-// items, numbered from w0 on, are FP32 blocks (a sub, a group of kSumRuns runs) or FP64 warps (a set
+// items, numbered from w0 on, are FP32 blocks (a sub, gps groups of kSumRuns runs) or FP64 warps (a set
 // of kSumJobs jobs, spw steps of 32 voxels); each writes one partial sum of its outputs.
 struct SumLevel {
   long long nvox;          // voxels summed by this call
@@ -143,6 +147,7 @@ struct SumLevel {
   int w0, units, splits;   // first item; items = units (subs or job sets) x splits
   int nblk_cap, nblk, vpb; // FP32: summation blocks (at most, now), voxels of one
   int nfull, ngf;          // FP32: whole runs per summation block, groups of whole runs
+  int ngrp, gps;           // FP32: groups, those of one block's partial sum
   int max_nf;              // FP32: most fields of a sub
   int spw, njobs;          // FP64: 32-voxel steps per warp, jobs
   const SumSub* subs;
@@ -152,7 +157,7 @@ struct SumLevel {
   const int* map;          // [n_ent] bin of each output (64 per tile, 4 per job), -1: none
   int n_ent, ent0;         // outputs, first output of the level in the launch
   double* partial;         // [splits][n_ent]
-  int rows;                // splits that fit `partial`
+  int rows;                // splits that fit `partial`; before it is allocated, those it is to fit at least
   double scale;            // msum = scale * sum
 };
 struct SumArgs {
