@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(256) reduce_sums_kernel(SumArgs a) {
 template <>
 bsp_status launch_contract_simt<float>(const SumArgs& a, cudaStream_t s) {
   if (a.items == 0) return BSP_OK;
-  BSP_CUDA(cudaFuncSetAttribute(contract_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem));
+  const bsp_status st = allow_shared(contract_f32_kernel, (size_t)sum_stage_bytes(kSumMaxFields));
+  if (st != BSP_OK) return st;
   contract_f32_kernel<<<a.items, kSumThreads, a.smem, s>>>(a);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;

@@ -468,7 +468,8 @@ namespace {
 template <int NP, int KT>
 bsp_status launch_tc(const TcArgs& a, const CUtensorMap* tmap, cudaStream_t s) {
   const int smem = TcLayout<NP, KT>::kBytes;
-  BSP_CUDA(cudaFuncSetAttribute(contract_tc_kernel<NP, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const bsp_status st = allow_shared(contract_tc_kernel<NP, KT>, (size_t)smem);
+  if (st != BSP_OK) return st;
   contract_tc_kernel<NP, KT><<<dim3(a.n_tg, a.gridy), tc_threads<KT>(), smem, s>>>(a, *tmap);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;

@@ -299,7 +299,9 @@ static bsp_status launch_pass(K kernel, const PassArgs& a, int n_items, int line
                               cudaStream_t s) {
   if (n_items == 0) return BSP_OK;
   const size_t smem = pass_smem<T>(lines, len, a.ngs);
-  BSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // a block's lines hold at most FftElems x kFftThreads points, a grid 4096
+  const bsp_status st = allow_shared(kernel, pass_smem<T>(1, FftElems<T>::value * kFftThreads, 4096));
+  if (st != BSP_OK) return st;
   kernel<<<n_items, kFftThreads, smem, s>>>(a, lines);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;

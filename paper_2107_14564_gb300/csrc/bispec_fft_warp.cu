@@ -788,7 +788,8 @@ template <int N, bool XPASS>
 bsp_status launch_xyf(const PassArgs& a, int n_items, float scale, cudaStream_t s) {
   if (n_items == 0) return BSP_OK;
   const size_t smem = ((size_t)N + (size_t)kLines * line_ld<N>() + (size_t)N * kTileLd) * sizeof(float2);
-  BSP_CUDA(cudaFuncSetAttribute(xyf_warp_kernel<N, XPASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const bsp_status st = allow_shared(xyf_warp_kernel<N, XPASS>, smem);
+  if (st != BSP_OK) return st;
   xyf_warp_kernel<N, XPASS><<<n_items, XY<N>::kThreads, smem, s>>>(a, scale);
   BSP_CUDA(cudaGetLastError());
   return BSP_OK;
@@ -798,7 +799,8 @@ template <int S>
 bsp_status launch_zf(const PassArgs& a, const float* gfield, long long n_lines, int n_sm, cudaStream_t s) {
   constexpr int LPW = 32 / Radices<S>::lpl;
   const size_t smem = ((size_t)S + (size_t)(kZThreads / 32) * LPW * z_line_ld<S>()) * sizeof(float2);
-  BSP_CUDA(cudaFuncSetAttribute(zf_warp_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const bsp_status st = allow_shared(zf_warp_kernel<S>, smem);
+  if (st != BSP_OK) return st;
   int per_sm = 0;
   BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, zf_warp_kernel<S>, kZThreads, smem));
   long long blocks = (long long)std::max(per_sm, 1) * n_sm;
@@ -816,7 +818,8 @@ bsp_status launch_xy(const PassArgs& a, int n_items, int n_sm, cudaStream_t s) {
   if constexpr (xy_in_lines(N, XPASS)) {
     const size_t smem = XYL<N>::kSmem;
     auto kern = xy_line_kernel<N, XPASS>;
-    BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const bsp_status st = allow_shared(kern, smem);
+    if (st != BSP_OK) return st;
     int per_sm = 0;
     BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, XYL<N>::kThreads, smem));
     constexpr int kUnits = XYL<N>::kThreads / 32;  // units of 4 lines a block takes at a time
@@ -830,7 +833,10 @@ bsp_status launch_xy(const PassArgs& a, int n_items, int n_sm, cudaStream_t s) {
   // two regions, each holding a tile of 2 r - 1 rows of the largest shell or, once it is read,
   // the line buffers
   const size_t smem = ((size_t)N + 2 * (size_t)xy_region<N>(a.rmax)) * sizeof(float2);
-  BSP_CUDA(cudaFuncSetAttribute(xy_warp_kernel<N, XPASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // modes stay below a third of the grid
+  const bsp_status st =
+      allow_shared(xy_warp_kernel<N, XPASS>, ((size_t)N + 2 * (size_t)xy_region<N>(N / 3 + 1)) * sizeof(float2));
+  if (st != BSP_OK) return st;
   int per_sm = 0;
   BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xy_warp_kernel<N, XPASS>, XY<N>::kThreads, smem));
   long long blocks = std::min<long long>((long long)std::max(per_sm, 1) * std::max(n_sm, 1), n_items);
@@ -845,10 +851,11 @@ template <int S>
 bsp_status launch_z(const PassArgs& a, long long n_lines, int n_sm, cudaStream_t s) {
   constexpr int M = S / 2;
   constexpr int LPW = 32 / Radices<M>::lpl;
-  const size_t smem = ((size_t)2 * M + (size_t)(kZThreads / 32) * LPW * z_line_ld<M>()) * sizeof(float2) +
-                      (a.n_zlev > 0 ? (size_t)S * sizeof(uint32_t) : 0);
+  const size_t lines = ((size_t)2 * M + (size_t)(kZThreads / 32) * LPW * z_line_ld<M>()) * sizeof(float2);
+  const size_t masks = (size_t)S * sizeof(uint32_t), smem = lines + (a.n_zlev > 0 ? masks : 0);
   auto kern = a.slab_nx > 0 ? z_warp_kernel<S, true> : z_warp_kernel<S, false>;
-  BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const bsp_status st = allow_shared(kern, lines + masks);
+  if (st != BSP_OK) return st;
   int per_sm = 0;
   BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kZThreads, smem));
   long long blocks = (long long)std::max(per_sm, 1) * n_sm;

@@ -132,7 +132,8 @@ bsp_status launch_adjoint(const float* fields, long long nvox, int ns, const int
   constexpr int VB = kAdjThreads * VPT;
   const size_t smem = (size_t)ns * VB * sizeof(float);
   auto kern = adjoint_products_kernel<NQ, VPT>;
-  BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const bsp_status st = allow_shared(kern, (size_t)4 * NQ * VB * sizeof(float));
+  if (st != BSP_OK) return st;
   int per_sm = 0;
   BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, smem));
   const long long blocks = std::min<long long>((nvox + VB - 1) / VB, (long long)std::max(per_sm, 1) * std::max(n_sm, 1) * 4);

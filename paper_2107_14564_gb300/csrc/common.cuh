@@ -184,6 +184,15 @@ bsp_status cuda_fail(cudaError_t e, const char* what);
     if (e_ != cudaSuccess) return ::bsp::cuda_fail(e_, #call); \
   } while (0)
 
+// Lets `kern` be launched with up to `most` bytes of dynamic shared memory. The limit is the process's, not the
+// launch's, so `most` depends on the kernel alone: were it the plan's size, another thread that
+// sets its own, smaller one between this call and the launch would have the launch refused.
+template <typename K>
+inline bsp_status allow_shared(K kern, size_t most) {
+  BSP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  return BSP_OK;
+}
+
 // ---------------------------------------------------------------- launchers (bispec_fft.cu)
 template <typename T>
 bsp_status launch_xpass(const PassArgs& a, int n_items, int lines, cudaStream_t s);
