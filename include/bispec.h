@@ -86,10 +86,10 @@ typedef struct {
                               plan-time counts and bsp_grad make the X and Y passes once and then
                               produce and reduce the fields one x-slab of the evaluation grid at a
                               time (the largest slab within the budget, sums added in FP64), on one
-                              contraction level. The X/Y pass buffers (rows of k_z padded to 8
+                              contraction level. Outside the budget are the X/Y pass buffers (FP32
+                              and mixed plans on grids of 128..1024 hold rows of k_z padded to 8
                               elements) and the contraction's partial sums (FP32: at most 60 MB a
-                              level) are outside the budget. A
-                              budget below one x-plane of all shells is BSP_ERR_INVALID_ARG;
+                              level). A budget below one x-plane of all shells is BSP_ERR_INVALID_ARG;
                               BSP_MIXED_BF16X3 plans whose fields exceed it need an evaluation grid
                               of 128..1024 points of the form 2^p or 3*2^p (else
                               BSP_ERR_NOT_SUPPORTED) and then hold one slab of split fields, so

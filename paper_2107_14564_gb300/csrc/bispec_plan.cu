@@ -734,7 +734,7 @@ bsp_status host_plan(bsp_plan* p, const bsp_plan_desc* d) {
     g.qlo = (int)p->q[n];
     g.qhi = (int)p->q[n + 1];
     g.r = (int)isqrt_ll(p->q[n + 1] - 1) + 1;
-    g.rp = row_pitch(g.r);
+    g.rp = p->dim == 2 || (p->prec != BSP_FP64 && warp_fft_supported(p->ngs)) ? row_pitch(g.r) : g.r;
     g.g1_off = o1;
     g.g2_off = o2;
     if (p->dim == 2) {  // one buffer of X-pass rows [x][k_y < r], read again by the C2R along y
