@@ -4,7 +4,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <functional>
 #include <new>
 #include <string>
 #include <vector>
@@ -121,56 +120,71 @@ static int count_pair_quads(const std::vector<int>& ta, const std::vector<int>& 
   return n;
 }
 
-// FP32 tables of a CUDA-core contraction level: tiles of 2 a x 4 (2) b x 8 (4) c taken off the bins from
+// FP32 tables of a CUDA-core contraction level: tiles of 2 a x 4 b x ncmax c taken off the bins from
 // the largest shells down, then blocks of `per` equally wide tiles that share fields, with the
-// fields they read. out[64 t + 32 i + 8 j + k]: the bin of output (i, j, k) of tile t.
+// fields they read. out[32 i + 8 j + k]: the bin of output (i, j, k) of a tile.
 struct SumRaw { int a[2], b[4], c[8], nc, out[64]; };
 static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std::vector<int>& tb,
                                           const std::vector<int>& tc, const std::vector<int>* ids, int ncmax) {
   std::vector<SumRaw> raw;
-  struct B { int a, b, c, id; };
-  std::vector<B> bins;
-  for (size_t t = 0; t < ta.size(); ++t) bins.push_back({ta[t], tb[t], tc[t], ids ? (*ids)[t] : (int)t});
-  auto distinct = [](std::vector<int> v) {  // descending
-    std::sort(v.begin(), v.end(), std::greater<int>());
+  struct Bin { int b, c, a, id; };  // a: 0 or 1, the place of its first shell in the tile
+  auto distinct = [](std::vector<int> v) {
+    std::sort(v.begin(), v.end());
     v.erase(std::unique(v.begin(), v.end()), v.end());
     return v;
   };
-  const std::vector<int> as = distinct(ta);
-  for (size_t i = 0; i < as.size(); i += 2) {
-    const int na = (int)std::min<size_t>(2, as.size() - i);
-    std::vector<B> sel;
-    std::vector<int> bs;
-    for (const B& x : bins)
-      if (x.a == as[i] || (na > 1 && x.a == as[i + 1])) { sel.push_back(x); bs.push_back(x.b); }
+  // the bins are sorted by a: those of one first shell are neighbours
+  std::vector<size_t> start;
+  for (size_t t = 0; t < ta.size(); ++t)
+    if (t == 0 || ta[t] != ta[t - 1]) start.push_back(t);
+  const size_t nas = start.size();
+  start.push_back(ta.size());
+  for (size_t i = 0; i < nas; i += 2) {  // first shells from the largest down
+    const int na = (int)std::min<size_t>(2, nas - i);
+    std::vector<Bin> sel;
+    std::vector<int> as, bs;
+    for (int k = 0; k < na; ++k) {
+      const size_t g = nas - 1 - i - k;
+      as.push_back(ta[start[g]]);
+      for (size_t t = start[g]; t < start[g + 1]; ++t) {
+        sel.push_back({tb[t], tc[t], k, ids ? (*ids)[t] : (int)t});
+        bs.push_back(tb[t]);
+      }
+    }
     bs = distinct(bs);
+    std::sort(sel.begin(), sel.end(), [](const Bin& x, const Bin& y) { return x.b != y.b ? x.b > y.b : x.c < y.c; });
+    size_t at = 0;  // first bin of the next four b
     for (size_t j = 0, nb; j < bs.size(); j += nb) {
       nb = std::min<size_t>(bs.size() - j, 4);
-      std::vector<B> rows;
+      size_t next[4], end[4];  // bins of each b not yet in a tile, ascending c
       std::vector<int> cs;
-      for (const B& x : sel)
-        for (size_t k = 0; k < nb; ++k)
-          if (x.b == bs[j + k]) { rows.push_back(x); cs.push_back(x.c); }
-      std::sort(cs.begin(), cs.end());
-      cs.erase(std::unique(cs.begin(), cs.end()), cs.end());
+      for (size_t k = 0; k < nb; ++k) {
+        next[k] = at;
+        while (at < sel.size() && sel[at].b == sel[next[k]].b) cs.push_back(sel[at++].c);
+        end[k] = at;
+      }
+      cs = distinct(cs);
       for (size_t m = 0, nc; m < cs.size(); m += nc) {
         nc = std::min<size_t>(cs.size() - m, ncmax);
         SumRaw t;
-        std::vector<int> ub;  // the b with a bin here
-        for (size_t k = 0; k < nb; ++k)
-          for (const B& x : rows)
-            if (x.b == bs[j + k] && x.c >= cs[m] && x.c <= cs[m + nc - 1]) { ub.push_back(x.b); break; }
+        for (int& o : t.out) o = -1;
+        int ub = 0;  // places taken: the b with a bin here
+        for (size_t k = 0; k < nb; ++k) {
+          bool any = false;
+          size_t ic = 0;
+          for (; next[k] < end[k] && sel[next[k]].c <= cs[m + nc - 1]; ++next[k]) {
+            const Bin& x = sel[next[k]];
+            while (cs[m + ic] != x.c) ++ic;
+            t.out[32 * x.a + 8 * ub + ic] = x.id;
+            any = true;
+          }
+          if (any) t.b[ub++] = sel[next[k] - 1].b;
+        }
         // places without a shell repeat the first
-        for (int k = 0; k < 2; ++k) t.a[k] = as[i + (k < na ? k : 0)];
-        for (size_t k = 0; k < 4; ++k) t.b[k] = ub[k < ub.size() ? k : 0];
+        for (int k = 0; k < 2; ++k) t.a[k] = as[k < na ? k : 0];
+        for (int k = ub; k < 4; ++k) t.b[k] = t.b[0];
         for (size_t k = 0; k < 8; ++k) t.c[k] = cs[m + (k < nc ? k : 0)];
         t.nc = nc > 4 ? 8 : 4;
-        for (int& o : t.out) o = -1;
-        for (const B& x : rows)
-          for (int ia = 0; ia < na; ++ia)
-            for (size_t ib = 0; ib < ub.size(); ++ib)
-              for (size_t ic = 0; ic < nc; ++ic)
-                if (x.a == t.a[ia] && x.b == t.b[ib] && x.c == t.c[ic]) t.out[32 * ia + 8 * ib + ic] = x.id;
         raw.push_back(t);
       }
     }
@@ -179,38 +193,50 @@ static std::vector<SumRaw> make_sum_tiles(const std::vector<int>& ta, const std:
   return raw;
 }
 
-static void make_sum_subs(std::vector<SumRaw> raw, int per, std::vector<SumTile>& tiles, std::vector<SumSub>& subs,
-                          std::vector<int>& sub_fields, std::vector<int>& map) {
-  while (!raw.empty()) {  // the first tile left, then those as wide that add the fewest fields
-    SumSub sub{(int)tiles.size(), 0, (int)sub_fields.size(), 0, raw.front().nc};
-    std::vector<int> cur;
-    auto with = [&](const SumRaw& t) {
-      std::vector<int> u = cur;
-      auto add = [&](const int* f, int n) {
-        for (int k = 0; k < n; ++k)
-          if (std::find(u.begin(), u.end(), f[k]) == u.end()) u.push_back(f[k]);
-      };
-      add(t.a, 2);
-      add(t.b, 4);
-      add(t.c, 8);
-      return u;
-    };
-    while (sub.ntiles < per && !raw.empty()) {
-      size_t best = 0, best_n = (size_t)-1;
-      for (size_t k = 0; k < raw.size() && raw[k].nc == sub.nc; ++k) {
-        const size_t n = with(raw[k]).size();
-        if (n < best_n) { best = k; best_n = n; }
-        if (cur.empty()) break;
+static void make_sum_subs(const std::vector<SumRaw>& raw, int per, std::vector<SumTile>& tiles,
+                          std::vector<SumSub>& subs, std::vector<int>& sub_fields, std::vector<int>& map) {
+  std::vector<int> left(raw.size());               // tiles without a block
+  std::vector<int> size(raw.size(), 0), lack;      // fields of each tile, those its block does not stage yet
+  std::vector<std::vector<int>> readers;           // tiles of each field
+  for (size_t i = 0; i < raw.size(); ++i) {
+    left[i] = (int)i;
+    auto reads = [&](const int* f, int n) {
+      for (int k = 0; k < n; ++k) {
+        if (readers.size() <= (size_t)f[k]) readers.resize(f[k] + 1);
+        std::vector<int>& r = readers[f[k]];
+        if (r.empty() || r.back() != (int)i) { r.push_back((int)i); ++size[i]; }
       }
-      if (best_n == (size_t)-1 || (!cur.empty() && best_n > (size_t)kSumMaxFields)) break;
-      const SumRaw t = raw[best];
-      raw.erase(raw.begin() + (long)best);
-      cur = with(t);
+    };
+    reads(raw[i].a, 2);
+    reads(raw[i].b, 4);
+    reads(raw[i].c, 8);
+  }
+  while (!left.empty()) {  // the first tile left, then those as wide that add the fewest fields
+    SumSub sub{(int)tiles.size(), 0, (int)sub_fields.size(), 0, raw[left[0]].nc};
+    std::vector<int> cur;
+    lack = size;
+    while (sub.ntiles < per && !left.empty()) {
+      size_t best = 0;
+      int least = kSumMaxFields + 1;
+      for (size_t k = 0; k < left.size() && raw[left[k]].nc == sub.nc; ++k) {
+        if (lack[left[k]] < least) { best = k; least = lack[left[k]]; }
+        if (cur.empty() || least == 0) break;  // the first one; none can add fewer
+      }
+      if ((int)cur.size() + least > kSumMaxFields) break;
+      const SumRaw& t = raw[left[best]];
+      left.erase(left.begin() + (long)best);
       SumTile s{};
-      auto at = [&](int f) { return (uint8_t)(std::find(cur.begin(), cur.end(), f) - cur.begin()); };
-      for (int k = 0; k < 2; ++k) s.a[k] = at(t.a[k]);
-      for (int k = 0; k < 4; ++k) s.b[k] = at(t.b[k]);
-      for (int k = 0; k < 8; ++k) s.c[k] = at(t.c[k]);
+      auto place = [&](int f) {
+        const size_t i = std::find(cur.begin(), cur.end(), f) - cur.begin();
+        if (i == cur.size()) {
+          cur.push_back(f);
+          for (int k : readers[f]) --lack[k];
+        }
+        return (uint8_t)i;
+      };
+      for (int k = 0; k < 2; ++k) s.a[k] = place(t.a[k]);
+      for (int k = 0; k < 4; ++k) s.b[k] = place(t.b[k]);
+      for (int k = 0; k < 8; ++k) s.c[k] = place(t.c[k]);
       tiles.push_back(s);
       map.insert(map.end(), t.out, t.out + 64);
       sub.ntiles += 1;
@@ -291,7 +317,7 @@ bsp_status make_sum_level(bsp_plan* p, const std::vector<int>& ta, const std::ve
     std::vector<SumTile> tiles;
     std::vector<SumSub> subs;
     std::vector<int> fields;
-    make_sum_subs(std::move(raw), per, tiles, subs, fields, map);
+    make_sum_subs(raw, per, tiles, subs, fields, map);
     SumTile* dt = nullptr;
     SumSub* ds = nullptr;
     int* df = nullptr;
