@@ -330,8 +330,8 @@ void stage_work(const bsp_plan* p, double* bytes, double* flops) {
   }
   // contraction levels, each pair on its smallest exact grid (a split-BF16 plan may contract some
   // pairs on a larger level where that is faster; that extra work is not counted): fields read
-  // once per level (lower levels also read their samples of the evaluation grid and write them),
-  // work per level on its g^3 grid
+  // once per level (split-BF16 plans also read the lower levels' samples of the evaluation grid and
+  // write them), work per level on its g^3 grid
   for (const auto& lv : p->exact_levels) {
     const int g = lv.first;
     const std::vector<int>& bins = lv.second;
@@ -350,7 +350,7 @@ void stage_work(const bsp_plan* p, double* bytes, double* flops) {
       const bsp_triplet& a = p->trips[bins[i]];
       if (i == 0 || a.a != p->trips[bins[i - 1]].a || a.b != p->trips[bins[i - 1]].b) npairs += 1;
     }
-    bytes[BSP_STAGE_CONTRACT] += re * nsh * nv * (top ? 1.0 : 3.0);
+    bytes[BSP_STAGE_CONTRACT] += re * nsh * nv * (top || p->prec != BSP_MIXED_BF16X3 ? 1.0 : 3.0);
     if (p->prec == BSP_MIXED_BF16X3)  // split-BF16 GEMM over the padded shell columns
       flops[BSP_STAGE_CONTRACT] += 3.0 * 2.0 * (double)npairs * (double)tc_padded_shells(nsh) * nv;
     else
