@@ -228,8 +228,9 @@ BSP_API bsp_status bsp_spectrum(bsp_plan* plan, const float* delta_x, void* spec
  *   G_n = sum_t dL/dB_t V_c^3 / (V T_t) (product of the bin's other two fields), one term per
  *   position of n in the bin, G^_n its forward DFT and K the Kaiser factor of Eq. (3.4).
  * Shell fields are recomputed (nothing is kept from a forward call); the first call allocates
- * the adjoint buffers (about two shell-field sets). FP32 and mixed plans whose grid sides are 2^p
- * or 3 * 2^p in [128, 1024]; else BSP_ERR_NOT_SUPPORTED. Asynchronous on `stream`. */
+ * the adjoint buffers (about two shell-field sets). FP32 and mixed plans of at most 64 shells whose
+ * grid sides are 2^p or 3 * 2^p in [128, 1024]; else BSP_ERR_NOT_SUPPORTED. Asynchronous on
+ * `stream`. */
 BSP_API bsp_status bsp_grad(bsp_plan* plan, const void* spec, const double* dl_db, float* dl_ddelta,
                             void* stream);
 

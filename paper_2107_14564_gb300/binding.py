@@ -306,7 +306,8 @@ class Plan:
         return spec
 
     def grad(self, spec: torch.Tensor, dl_db: torch.Tensor, stream=None) -> torch.Tensor:
-        """dL/d delta(x) on the Ng^3 grid for dl_db = dL/dB per kept bin (float32 CUDA tensor)."""
+        """dL/d delta(x) on the Ng^3 grid for dl_db = dL/dB per kept bin (float32 CUDA tensor); at most
+        64 shells."""
         self._check_spec(spec)
         g = dl_db.to(device=spec.device, dtype=torch.float64).contiguous()
         if g.numel() != self.n_triplets:
