@@ -38,9 +38,8 @@ constexpr int kSumQuads = kSumVox / 4;
 constexpr int kSumRow = 4 * kSumVox;          // bytes of a run in a staged field
 constexpr int kSumFieldBytes = 32 * kSumRow;  // one field of a stage: 32 runs
 // Run r's quad q lies in place q ^ sum_swz(r): eight lanes' 16-byte reads of one field meet all banks.
-__host__ __device__ constexpr int sum_swz(int r) {
-  return (r >> (kSumVox == 8 ? 2 : kSumVox == 16 ? 1 : 0)) & (kSumQuads - 1);
-}
+static_assert(kSumRow == 128, "a run's stage is one row of all banks");
+__host__ __device__ constexpr int sum_swz(int r) { return r & (kSumQuads - 1); }
 constexpr int kF64Warps = 4;
 constexpr int kF64Run = 64;  // 32-voxel steps summed lane by lane
 

@@ -24,10 +24,12 @@
 //     voxels of every K step. It loads its slot's fields from shared memory, forms the products
 //     in bf16x2 arithmetic and writes them into the tensor-memory A stage of each tile with
 //     tcgen05.st .16x256b (whose lane map puts a thread's registers in rows r and r + 8). A warp
-//     takes every other chunk whole (all 4 K steps): it hands its last chunk's stage over while
-//     this chunk's loads are in flight, forms the products and only then waits for the MMAs of
-//     chunk i - NA to free its A stage. Half of each chunk per warp instead paid the stage
-//     hand-over and the waits twice as often (3.39 -> 3.35 ms at Ng = 512 and 32 shells).
+//     takes every other chunk whole (all 4 K steps): it forms the first two K steps' products, waits
+//     for the MMAs of chunk i - NA to free its A stage, stores them, does the other two, waits for its
+//     own stores and hands the stage over before it turns to its next chunk; the warps of the
+//     other parity work meanwhile. Half of each chunk per warp instead, with the hand-over put off until
+//     the next chunk's loads were in flight, paid it and the waits twice as often (3.39 -> 3.35 ms at
+//     Ng = 512 and 32 shells).
 //   * KT MMA warps, one per tile: one thread issues the tile's 4 MMAs of a chunk into its FP32
 //     accumulator and commits them to the B stage's "mma done" mbarrier (KT arrivals), which frees
 //     the B stage for the loader and (NA chunks later) the A stage for the generators. One
@@ -127,6 +129,7 @@ struct Sum2 {
   }
 };
 
+// No instance spills but <64, 2> (4 bytes).
 template <int NP, int KT>
 __global__ void __launch_bounds__(tc_threads<KT>(), 1)
     contract_tc_kernel(TcArgs a, const __grid_constant__ CUtensorMap tmap) {

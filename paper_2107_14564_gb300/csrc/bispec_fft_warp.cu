@@ -380,7 +380,8 @@ template <int N> struct XYL {
   static constexpr int kLen = N + N / kR0;
   static constexpr int kLd = kLen + (20 - kLen % 16) % 16;
   static constexpr int kThreads = 128;
-  static constexpr int kBlocks = N <= 128 ? 6 : N <= 192 ? 5 : N <= 256 ? 4 : 3;  // as the points' registers allow
+  // as the points' registers allow (8 bytes of the X pass at 192 points spill)
+  static constexpr int kBlocks = N <= 128 ? 6 : N <= 192 ? 5 : N <= 256 ? 4 : 3;
   static constexpr size_t kSmem = ((size_t)N + (size_t)(kThreads / 32) * 4 * kLd) * sizeof(float2);
 };
 
@@ -830,20 +831,20 @@ bsp_status launch_xy(const PassArgs& a, int n_items, int n_sm, cudaStream_t s) {
     BSP_CUDA(cudaGetLastError());
     return BSP_OK;
   } else {
-  // two regions, each holding a tile of 2 r - 1 rows of the largest shell or, once it is read,
-  // the line buffers
-  const size_t smem = ((size_t)N + 2 * (size_t)xy_region<N>(a.rmax)) * sizeof(float2);
-  // modes stay below a third of the grid
-  const bsp_status st =
-      allow_shared(xy_warp_kernel<N, XPASS>, ((size_t)N + 2 * (size_t)xy_region<N>(N / 3 + 1)) * sizeof(float2));
-  if (st != BSP_OK) return st;
-  int per_sm = 0;
-  BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xy_warp_kernel<N, XPASS>, XY<N>::kThreads, smem));
-  long long blocks = std::min<long long>((long long)std::max(per_sm, 1) * std::max(n_sm, 1), n_items);
-  if (!XPASS && a.grid_blocks > 0) blocks = std::min<long long>(a.grid_blocks, n_items);
-  xy_warp_kernel<N, XPASS><<<(unsigned)blocks, XY<N>::kThreads, smem, s>>>(a, n_items);
-  BSP_CUDA(cudaGetLastError());
-  return BSP_OK;
+    // two regions, each holding a tile of 2 r - 1 rows of the largest shell or, once it is read,
+    // the line buffers
+    const size_t smem = ((size_t)N + 2 * (size_t)xy_region<N>(a.rmax)) * sizeof(float2);
+    // modes stay below a third of the grid
+    const bsp_status st =
+        allow_shared(xy_warp_kernel<N, XPASS>, ((size_t)N + 2 * (size_t)xy_region<N>(N / 3 + 1)) * sizeof(float2));
+    if (st != BSP_OK) return st;
+    int per_sm = 0;
+    BSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xy_warp_kernel<N, XPASS>, XY<N>::kThreads, smem));
+    long long blocks = std::min<long long>((long long)std::max(per_sm, 1) * std::max(n_sm, 1), n_items);
+    if (!XPASS && a.grid_blocks > 0) blocks = std::min<long long>(a.grid_blocks, n_items);
+    xy_warp_kernel<N, XPASS><<<(unsigned)blocks, XY<N>::kThreads, smem, s>>>(a, n_items);
+    BSP_CUDA(cudaGetLastError());
+    return BSP_OK;
   }
 }
 
