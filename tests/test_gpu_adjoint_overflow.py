@@ -25,7 +25,7 @@ def test_adjoint_takes_no_product_outside_the_bins():
     shell = P.shell_index_half(pl)
     amp = np.choose(shell.clip(0), (2e21, 1e12, 1e12)) * (shell >= 0)
     spec = amp * (rng.standard_normal(shell.shape) + 1j * rng.standard_normal(shell.shape))
-    delta = np.fft.irfftn(spec, s=(ng,) * 3)
+    delta = np.fft.irfftn(spec, s=(ng,) * 3, axes=(0, 1, 2))
     spec = np.fft.rfftn(delta)
     g = rng.standard_normal(len(trips))
     want = G.vjp(delta, pl, trips, gp.triplets["tsum"], g)
