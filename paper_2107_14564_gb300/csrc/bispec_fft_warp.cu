@@ -50,8 +50,8 @@ template <> struct Radices<1024> { static constexpr int lpl = 32, n = 4; static 
 //     ns R points put the runs side by side;
 //   * later exchanges move whole half-warps.
 // All of it folds into constants, the lane's own part aside. One padding for every exchange of a
-// length left 25% (192, 256) to 100% (96) more wavefronts, and these passes are bound by that pipe (Z
-// 97% busy): estimates at Ng = 256 and 24 shells 1.53 -> 1.48 ms (FP32), 0.957 -> 0.907 (split BF16, host
+// length left 25% (192, 256) to 100% (96) more wavefronts, and these passes are bound by that pipe (Z of
+// 192-point lines 97% busy then, 89% now): estimates at Ng = 256 and 24 shells 1.53 -> 1.48 ms (FP32), 0.957 -> 0.907 (split BF16, host
 // buffers), the shell fields at Ng = 384 and 8 shells 847 -> 818 us. XOR permutations without
 // conflicts cost more address arithmetic than they saved at 192 points (868 us).
 // The X/Y passes keep one placement from 384 points on, where longer lines would cost resident

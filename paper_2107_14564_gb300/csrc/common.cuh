@@ -135,7 +135,9 @@ constexpr int kSumRun = 1024;     // voxels of one FP32 accumulation run
 constexpr int kSumJobs = 8;       // FP64 jobs of a warp
 // FP32 blocks of a level per SM above which a block takes several groups: partial sums, one row a block,
 // stay within 64 x SMs x kSumWarps x 64 doubles (60 MB) whatever the voxels, and the last wave
-// within 1/32 of the time.
+// within 1/32 of the time. A row per group took 0.9 GB at Ng = 512 and 64 shells and 95.4 ms an estimate, now
+// 94.4 (fewer rows to write and add); Ng = 768, 24 shells in x-slabs 88.1 -> 87.7 ms. Levels below the line
+// (up to Ng = 256 at 24 shells) keep a block per group.
 constexpr int kSumWaves = 64;
 
 // One level of a CUDA-core contraction launch: triple sums over the g^3 voxels sampled from source
